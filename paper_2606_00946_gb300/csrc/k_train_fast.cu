@@ -44,7 +44,9 @@ enum { TE_STORE = 0, TE_FWD = 1, TE_FWD_OUT = 2, TE_DX = 3 };
 // split), so the column parts of a tile are adjacent (a cluster for TE_FWD_OUT).
 struct TrJob {
   int epi;
-  int m_tiles, n_split, splits, nchunks;
+  int m_tiles, n_split, splits;
+  int nchunks;                       // K-blocks of 64 per CTA (the last split may hold fewer)
+  int kblocks;                       // K-blocks of the whole product
   int NT;                            // columns per CTA; the product's N = NT * n_split
   const uint8_t* A;                  // image, rA rows
   int rA;
@@ -76,6 +78,12 @@ struct TrJob {
   // the dropped activation drop_h (its keep bits are in mask_in)
   int drop_h;
 };
+
+// K-blocks of split `split` of job J: splits hold nchunks each, the last what
+// is left of the product's kblocks.
+__device__ __forceinline__ int tr_chunks(const TrJob& J, int split) {
+  return min(J.nchunks, J.kblocks - split * J.nchunks);
+}
 
 struct TrArgs {
   TrJob job[2];
@@ -198,7 +206,7 @@ __device__ __forceinline__ void tr_tile_pre(const TrArgs& args, int bid, uint8_t
   const int li = second ? bid - args.n_cta0 : bid;
   const int ns = li % J.n_split, rest = li / J.n_split;
   const int split = rest / J.m_tiles;
-  const int NT = J.NT, N = NT * J.n_split, n0 = ns * NT, nch = J.nchunks;
+  const int NT = J.NT, N = NT * J.n_split, n0 = ns * NT, nch = tr_chunks(J, split);
   const uint32_t a_bytes = kM * 128, b_bytes = (uint32_t)NT * 128;
   const uint32_t stage_bytes = a_bytes + b_bytes;
   uint8_t* tail = tr_tail(smem);
@@ -209,7 +217,7 @@ __device__ __forceinline__ void tr_tile_pre(const TrArgs& args, int bid, uint8_t
   if (tid == 0) {
     const bool b_static = J.epi != TE_STORE;  // the weight-gradient products read activations
     for (int c = 0; c < nch; ++c) {
-      const int kb = split * nch + c;
+      const int kb = split * J.nchunks + c;
       mbar_arrive_expect_tx(&full[c], stage_bytes);
       if (b_static) bulk_g2s(smem + (size_t)c * stage_bytes + a_bytes, J.B + (size_t)kb * N * 128 + (size_t)n0 * 128,
                              b_bytes, &full[c]);
@@ -232,12 +240,12 @@ __device__ __forceinline__ void tr_tile_copies(const TrArgs& args, int bid, uint
   const int ns = li % J.n_split, rest = li / J.n_split;
   const int mt = rest % J.m_tiles, split = rest / J.m_tiles;
   const int m0 = mt * kM;
-  const int NT = J.NT, N = NT * J.n_split, n0 = ns * NT, nch = J.nchunks;
+  const int NT = J.NT, N = NT * J.n_split, n0 = ns * NT, nch = tr_chunks(J, split);
   const uint32_t a_bytes = kM * 128, b_bytes = (uint32_t)NT * 128;
   const uint32_t stage_bytes = a_bytes + b_bytes;
   uint64_t* full = reinterpret_cast<uint64_t*>(tr_tail(smem));
   for (int c = 0; c < nch; ++c) {
-    const int kb = split * nch + c;
+    const int kb = split * J.nchunks + c;
     uint8_t* sa = smem + (size_t)c * stage_bytes;
     bulk_g2s(sa, J.A + (size_t)kb * J.rA * 128 + (size_t)m0 * 128, a_bytes, &full[c]);
     if (J.epi == TE_STORE) bulk_g2s(sa + a_bytes, J.B + (size_t)kb * N * 128 + (size_t)n0 * 128, b_bytes, &full[c]);
@@ -259,7 +267,7 @@ __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* sm
   const int ns = li % J.n_split, rest = li / J.n_split;
   const int mt = rest % J.m_tiles, split = rest / J.m_tiles;
   const int m0 = mt * kM;
-  const int NT = J.NT, N = NT * J.n_split, n0 = ns * NT, nch = J.nchunks;
+  const int NT = J.NT, N = NT * J.n_split, n0 = ns * NT, nch = tr_chunks(J, split);
   const uint32_t a_bytes = kM * 128, b_bytes = (uint32_t)NT * 128;
   const uint32_t stage_bytes = a_bytes + b_bytes;
   uint8_t* tail = tr_tail(smem);
@@ -1100,7 +1108,7 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
     // batch of 4096: half the epilogue and image stores per SM)
     J.n_split = (last && one) ? 1 : (!last && !one && m.w[l + 1] % 256 == 0) ? 4 : n_split_for(m.w[l + 1]);
     J.splits = 1;
-    J.nchunks = f.in_pad[l] / 64;
+    J.nchunks = J.kblocks = f.in_pad[l] / 64;
     J.NT = m.w[l + 1] / J.n_split;
     J.A = f.imgA[l];
     J.rA = R;
@@ -1145,8 +1153,9 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
     // K-blocks (of 64 batch rows) per CTA: 4 when that still gives 48 CTAs,
     // else 2 (more CTAs, more partials for the optimiser to add)
     const int kpc = W.m_tiles * W.n_split * (R / 256) >= 48 ? 4 : 2;
-    W.nchunks = std::min(kpc, R / 64);
-    W.splits = (R / 64) / W.nchunks;
+    W.kblocks = R / 64;
+    W.nchunks = std::min(kpc, W.kblocks);
+    W.splits = (W.kblocks + W.nchunks - 1) / W.nchunks;  // the last one may be short
     W.NT = f.in_pad[l] / W.n_split;
     W.A = f.imgDZT[l & 1];
     W.rA = ((out + 127) / 128) * 128;
@@ -1162,7 +1171,7 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
       X.m_tiles = T;
       X.n_split = n_split_for(m.w[l]);
       X.splits = 1;
-      X.nchunks = out / 64;
+      X.nchunks = X.kblocks = out / 64;
       X.NT = m.w[l] / X.n_split;
       X.A = f.imgDZ[l & 1];
       X.rA = R;
