@@ -283,7 +283,7 @@ int ls_create(const ls_config* cfg, ls_ctx** out) {
   A(dalloc(&c.st, 1));
   int64_t tf_bytes = 0;
   const bool fast_train = plan_train_fast(m, cfg->max_train_batch, c.tf);
-  if (cfg->dropout > 0.0f && !fast_train) {
+  if (cfg->dropout > 0.0f && (!fast_train || c.tf.wide)) {
     free_all(c);
     delete h;
     return fail(LS_ERR_ARG, "dropout needs the tensor-core training path (bf16, hidden widths <= 256)");
@@ -295,7 +295,7 @@ int ls_create(const ls_config* cfg, ls_ctx** out) {
     A(dalloc(&c.tf.parts, pf));
     A(dalloc(&c.tr_bar, 2));
     if (e == cudaSuccess) train_fast_bind(m, c.tf, c.tf.base, c.tf.parts);
-    c.train_ctas = cfg->train_ctas > 0 ? std::min(cfg->train_ctas, c.sms) : 0;
+    c.train_ctas = cfg->train_ctas > 0 && !c.tf.wide ? std::min(cfg->train_ctas, c.sms) : 0;
   }
   if (e == cudaSuccess) {
     A(cudaEventCreateWithFlags(&c.ev_pub, cudaEventDisableTiming));

@@ -167,6 +167,7 @@ struct Tracer {
 // fp32 partials the optimiser sums.
 struct TrainFast {
   bool on = false;
+  bool wide = false;                       // a hidden layer wider than 256 (chained launches only, no dropout)
   int rows_max = 0;                        // max_train_batch rounded up to 128
   int in_pad[LS_MAX_LAYERS] = {};          // K of layer l (input width padded to 64)
   uint8_t* imgA[LS_MAX_LAYERS] = {};       // A_l  [rows, in_pad[l]]

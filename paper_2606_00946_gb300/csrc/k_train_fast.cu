@@ -35,7 +35,9 @@ namespace {
 
 constexpr int kT = 512;        // 16 warps: TMEM lane quadrant = warp % 4, column quarter = warp / 4
 constexpr int kM = 128;        // rows per tile
-constexpr int kMaxChunks = 4;  // K-blocks of 64 per CTA (all resident)
+constexpr int kMaxChunks = 8;  // K-blocks of 64 per CTA
+constexpr int kStageRegion = 4 * (kM * 128 + 256 * 128);  // operand stages (as many as fit, at least four)
+constexpr int kTailBar = 256;  // barriers and the TMEM address, before the epilogue scratch
 
 enum { TE_STORE = 0, TE_FWD = 1, TE_FWD_OUT = 2, TE_DX = 3 };
 
@@ -47,6 +49,7 @@ struct TrJob {
   int m_tiles, n_split, splits;
   int nchunks;                       // K-blocks of 64 per CTA (the last split may hold fewer)
   int kblocks;                       // K-blocks of the whole product
+  int stages;                        // tr_stages(NT)
   int NT;                            // columns per CTA; the product's N = NT * n_split
   const uint8_t* A;                  // image, rA rows
   int rA;
@@ -84,6 +87,11 @@ struct TrJob {
 __device__ __forceinline__ int tr_chunks(const TrJob& J, int split) {
   return min(J.nchunks, J.kblocks - split * J.nchunks);
 }
+
+// Operand stages a product with NT columns per CTA has (a stage: the 128-row
+// A tile and the NT-row B tile of one K-block).  With more K-blocks than
+// stages, K-block c + stages refills the stage of K-block c.
+int tr_stages(int NT) { return std::min(kMaxChunks, kStageRegion / (kM * 128 + NT * 128)); }
 
 struct TrArgs {
   TrJob job[2];
@@ -187,42 +195,52 @@ __device__ __forceinline__ void fwd_cols(uint32_t taddr, const float* s_bias, in
   }
 }
 
-// Shared memory of a training-product CTA: kMaxChunks stages of one 128-row A
-// tile and one (<= 256)-row B tile, then the barriers and epilogue scratch.
-__device__ __forceinline__ uint8_t* tr_tail(uint8_t* smem) {
-  return smem + (size_t)kMaxChunks * (kM * 128 + 256 * 128);
+// Shared memory of a training-product CTA: the operand stages, then the
+// barriers (kMaxChunks `full`, `done`, kMaxChunks `used`) and epilogue scratch.
+__device__ __forceinline__ uint8_t* tr_tail(uint8_t* smem) { return smem + kStageRegion; }
+
+// The copy of K-block c's operands (`a`: the 128-row tile of A, `b`: the
+// columns of B) into stage s.
+__device__ __forceinline__ void tr_copy(const TrJob& J, int c, int s, int kb, int m0, int n0, bool a, bool b, uint8_t* smem,
+                                        uint64_t* full) {
+  const int NT = J.NT, N = NT * J.n_split;
+  const uint32_t a_bytes = kM * 128, b_bytes = (uint32_t)NT * 128;
+  uint8_t* st = smem + (size_t)s * (a_bytes + b_bytes);
+  if (a) bulk_g2s(st, J.A + (size_t)kb * J.rA * 128 + (size_t)m0 * 128, a_bytes, &full[c]);
+  if (b) bulk_g2s(st + a_bytes, J.B + (size_t)kb * N * 128 + (size_t)n0 * 128, b_bytes, &full[c]);
 }
 
 // The part of tile `bid` that reads nothing the step's earlier products
-// write: arm every chunk barrier for the tile (the chunk barriers it does not
-// use are arrived on with no bytes, so each advances one phase per tile),
+// write: arm the tile's chunk barriers (for a CTA that runs `many` tiles, the
+// barriers it does not use are arrived on with no bytes, so each advances one
+// phase per tile),
 // copy the weight operand (forward and input-gradient products read the
 // weight images, which only the optimiser of the previous step writes) and
 // stage the epilogue's bias and output weights (the fp32 master).  A
 // per-launch product runs it before waiting for its predecessor.
-__device__ __forceinline__ void tr_tile_pre(const TrArgs& args, int bid, uint8_t* smem) {
+template <bool RING>
+__device__ __forceinline__ void tr_tile_pre(const TrArgs& args, int bid, uint8_t* smem, bool many) {
   const bool second = bid >= args.n_cta0;
   const TrJob& J = args.job[second ? 1 : 0];
   const int li = second ? bid - args.n_cta0 : bid;
   const int ns = li % J.n_split, rest = li / J.n_split;
   const int split = rest / J.m_tiles;
-  const int NT = J.NT, N = NT * J.n_split, n0 = ns * NT, nch = tr_chunks(J, split);
-  const uint32_t a_bytes = kM * 128, b_bytes = (uint32_t)NT * 128;
-  const uint32_t stage_bytes = a_bytes + b_bytes;
+  const int NT = J.NT, n0 = ns * NT, nch = tr_chunks(J, split);
+  const uint32_t stage_bytes = kM * 128 + (uint32_t)NT * 128;
   uint8_t* tail = tr_tail(smem);
   uint64_t* full = reinterpret_cast<uint64_t*>(tail);
-  float* s_bias = reinterpret_cast<float*>(tail + 128);
+  float* s_bias = reinterpret_cast<float*>(tail + kTailBar);
   float* s_w = s_bias + 256;
   const int tid = threadIdx.x;
   if (tid == 0) {
     const bool b_static = J.epi != TE_STORE;  // the weight-gradient products read activations
+    const int S = RING ? J.stages : kMaxChunks;
     for (int c = 0; c < nch; ++c) {
-      const int kb = split * J.nchunks + c;
       mbar_arrive_expect_tx(&full[c], stage_bytes);
-      if (b_static) bulk_g2s(smem + (size_t)c * stage_bytes + a_bytes, J.B + (size_t)kb * N * 128 + (size_t)n0 * 128,
-                             b_bytes, &full[c]);
+      if (b_static && c < S) tr_copy(J, c, c, split * J.nchunks + c, 0, n0, false, true, smem, full);
     }
-    for (int c = nch; c < kMaxChunks; ++c) mbar_arrive(&full[c]);
+    if (many)
+      for (int c = nch; c < kMaxChunks; ++c) mbar_arrive(&full[c]);
   }
   for (int t = tid; t < NT; t += kT) {
     if (J.bias) s_bias[t] = __ldg(J.bias + n0 + t);
@@ -233,6 +251,7 @@ __device__ __forceinline__ void tr_tile_pre(const TrArgs& args, int bid, uint8_t
 // The operand copies of tile `bid` that tr_tile_pre left (the activation or
 // gradient operand; both operands of a weight-gradient product), by one
 // thread, onto the barriers tr_tile_pre armed.
+template <bool RING>
 __device__ __forceinline__ void tr_tile_copies(const TrArgs& args, int bid, uint8_t* smem) {
   const bool second = bid >= args.n_cta0;
   const TrJob& J = args.job[second ? 1 : 0];
@@ -240,16 +259,11 @@ __device__ __forceinline__ void tr_tile_copies(const TrArgs& args, int bid, uint
   const int ns = li % J.n_split, rest = li / J.n_split;
   const int mt = rest % J.m_tiles, split = rest / J.m_tiles;
   const int m0 = mt * kM;
-  const int NT = J.NT, N = NT * J.n_split, n0 = ns * NT, nch = tr_chunks(J, split);
-  const uint32_t a_bytes = kM * 128, b_bytes = (uint32_t)NT * 128;
-  const uint32_t stage_bytes = a_bytes + b_bytes;
+  const int NT = J.NT, n0 = ns * NT;
+  const int nch = RING ? min(tr_chunks(J, split), J.stages) : tr_chunks(J, split);
   uint64_t* full = reinterpret_cast<uint64_t*>(tr_tail(smem));
-  for (int c = 0; c < nch; ++c) {
-    const int kb = split * J.nchunks + c;
-    uint8_t* sa = smem + (size_t)c * stage_bytes;
-    bulk_g2s(sa, J.A + (size_t)kb * J.rA * 128 + (size_t)m0 * 128, a_bytes, &full[c]);
-    if (J.epi == TE_STORE) bulk_g2s(sa + a_bytes, J.B + (size_t)kb * N * 128 + (size_t)n0 * 128, b_bytes, &full[c]);
-  }
+  for (int c = 0; c < nch; ++c)
+    tr_copy(J, c, c, split * J.nchunks + c, m0, n0, true, J.epi == TE_STORE, smem, full);
 }
 
 // One output tile (part `bid` of the products in `args`) on this CTA's shared
@@ -259,6 +273,7 @@ __device__ __forceinline__ void tr_tile_copies(const TrArgs& args, int bid, uint
 // the tile's image stores to reach global memory (other CTAs of the grid read
 // them); otherwise only until they have read shared memory.  Returns false
 // after a timed-out wait (error latched, copies in flight waited for).
+template <bool RING>
 __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* smem, uint32_t tmem, uint32_t par,
                                         bool drain, bool copied) {
   const bool second = bid >= args.n_cta0;
@@ -273,7 +288,8 @@ __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* sm
   uint8_t* tail = tr_tail(smem);
   uint64_t* full = reinterpret_cast<uint64_t*>(tail);           // [kMaxChunks]
   uint64_t* done = full + kMaxChunks;
-  float* s_bias = reinterpret_cast<float*>(tail + 128);         // [256]
+  uint64_t* used = done + 1;                                    // [kMaxChunks] K-block read by the products
+  float* s_bias = reinterpret_cast<float*>(tail + kTailBar);    // [256]
   float* s_w = s_bias + 256;                                    // [256] bf16-rounded output weights
   float* red = s_w + 256;                                       // [4][256] column sums by lane quadrant
   float* red2 = red + 4 * 256;                                  // [4][256]
@@ -283,17 +299,31 @@ __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* sm
   float* wsum = yrow + 128;                                     // [8] warp partials
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int S = RING ? J.stages : kMaxChunks;
+  int copies = min(nch, S);  // K-blocks whose copies were issued (thread 0)
   bool ok = true;
   if (tid == 0) {
-    if (!copied) tr_tile_copies(args, bid, smem);
+    if (!copied) tr_tile_copies<RING>(args, bid, smem);
     const uint32_t idesc = idesc_bf16_f32(kM, NT);
+    // RING (hidden layers wider than 256, one tile per launch): there may be
+    // more K-blocks than stages, at most twice as many
     for (int c = 0; c < nch; ++c) {
       if (!mbar_wait(&full[c], par)) { ok = false; break; }
       tc_fence_after();
-      const uint32_t sa = smem_u32(smem + (size_t)c * stage_bytes), sb = sa + a_bytes;
+      const uint32_t sa = smem_u32(smem + (size_t)(c < S ? c : c - S) * stage_bytes), sb = sa + a_bytes;
 #pragma unroll
       for (int k = 0; k < 4; ++k)
         umma_bf16(tmem, sdesc_sw128(sa + 32u * k), sdesc_sw128(sb + 32u * k), idesc, (c | k) ? 1u : 0u);
+      if (RING) {
+        // refill the previous K-block's stage once its products have read it
+        // (this K-block's products keep the tensor core busy meanwhile)
+        if (c + S < nch) umma_commit(&used[c]);
+        if (c >= 1 && c - 1 + S < nch) {
+          if (!mbar_wait(&used[c - 1], 0)) { ok = false; break; }
+          tr_copy(J, c - 1 + S, c - 1, split * J.nchunks + c - 1 + S, m0, n0, true, true, smem, full);
+          copies = c + S;
+        }
+      }
     }
     umma_commit(done);  // arrives once everything issued so far has completed
   }
@@ -305,7 +335,7 @@ __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* sm
     // copies that may still be in flight land in this CTA's own shared memory;
     // wait (bounded) for them before the CTA exits
     if (tid == 0)
-      for (int c = 0; c < nch; ++c) mbar_wait(&full[c], par);
+      for (int c = 0; c < copies; ++c) mbar_wait(&full[c], par);
   }
   tc_fence_after();
 
@@ -404,14 +434,21 @@ __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* sm
     else __syncthreads();
     if (ok && tid < kM) {
       float tot = rowdot[tid];
-      if (J.n_split > 1) {
-        const uint32_t me = cluster_ctarank();
-        const float other = ld_dsmem_f32(rowdot + tid, me ^ 1u);
-        tot = me == 0 ? tot + other : other + tot;  // rank 0's part first on both
+      if (J.n_split > 1) {  // the ranks' parts in rank order on every rank
+        if (!RING || J.n_split == 2) {
+          const uint32_t me = cluster_ctarank();
+          const float other = ld_dsmem_f32(rowdot + tid, me ^ 1u);
+          tot = me == 0 ? tot + other : other + tot;
+        } else {  // four
+          float v[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) v[k] = ld_dsmem_f32(rowdot + tid, (uint32_t)k);
+          tot = ((v[0] + v[1]) + v[2]) + v[3];
+        }
       }
       yrow[tid] = tot + __ldg(J.bL);
     }
-    if (J.n_split > 1) cluster_sync();  // the partner has read this CTA's rowdot
+    if (J.n_split > 1) cluster_sync();  // the other ranks have read this CTA's rowdot
     else __syncthreads();
     if (ok) {
       const bool valid = j < J.batch;
@@ -488,16 +525,23 @@ __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* sm
 }
 
 // One launch per product (or pair of products): CTA b runs tile b.
+template <bool RING>
 __global__ void __launch_bounds__(kT, 1) k_tr_gemm(const __grid_constant__ TrArgs args) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* full = reinterpret_cast<uint64_t*>(tr_tail(smem));
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(full + kMaxChunks + 1);
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(full + 2 * kMaxChunks + 1);
   const int NT = args.job[(int)blockIdx.x >= args.n_cta0 ? 1 : 0].NT;
   uint32_t tcols = 32;
   while ((int)tcols < NT) tcols <<= 1;
   if (threadIdx.x == 0) {
-    for (int c = 0; c <= kMaxChunks; ++c) mbar_init(&full[c], 1);  // chunk barriers, then `done`
+    // `full` of the tile's K-blocks, `done`, and `used` of those refilled (one
+    // thread sets them up one after the other, so only what the tile needs)
+    const TrJob& J = args.job[(int)blockIdx.x >= args.n_cta0 ? 1 : 0];
+    for (int c = 0; c < J.nchunks; ++c) mbar_init(&full[c], 1);
+    mbar_init(&full[kMaxChunks], 1);
+    if (RING)
+      for (int c = J.stages; c < J.nchunks; ++c) mbar_init(&full[kMaxChunks + 1 + c - J.stages], 1);
     fence_mbar_init();
   }
   if (threadIdx.x < 32) {
@@ -511,18 +555,18 @@ __global__ void __launch_bounds__(kT, 1) k_tr_gemm(const __grid_constant__ TrArg
   // optimiser has completed: the weight images and the master read before
   // the wait below are final.
   pdl_trigger();
-  tr_tile_pre(args, (int)blockIdx.x, smem);
+  tr_tile_pre<RING>(args, (int)blockIdx.x, smem, false);
   // the activation and gradient operands come from the previous kernels of the
   // stream: their copies start as soon as the wait returns
   pdl_wait();
-  if (threadIdx.x == 0) tr_tile_copies(args, (int)blockIdx.x, smem);
+  if (threadIdx.x == 0) tr_tile_copies<RING>(args, (int)blockIdx.x, smem);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_holder;
   // image stores may still be in flight when the CTA exits: the grid's
   // completion makes them visible to the next kernel
-  tr_tile(args, (int)blockIdx.x, smem, tmem, 0, false, true);
+  tr_tile<RING>(args, (int)blockIdx.x, smem, tmem, 0, false, true);
   if (threadIdx.x < 32) tmem_dealloc(tmem, tcols);
 }
 
@@ -851,10 +895,10 @@ __global__ void __launch_bounds__(kT, 1) k_tr_step(const __grid_constant__ StepA
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* full = reinterpret_cast<uint64_t*>(tr_tail(smem));
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(full + kMaxChunks + 1);
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(full + 2 * kMaxChunks + 1);
   const int tid = threadIdx.x;
   if (tid == 0) {
-    for (int c = 0; c <= kMaxChunks; ++c) mbar_init(&full[c], 1);  // chunk barriers, then `done`
+    for (int c = 0; c <= 2 * kMaxChunks; ++c) mbar_init(&full[c], 1);  // `full`, `done`, `used`
     fence_mbar_init();
   }
   if (tid < 32) {
@@ -874,8 +918,8 @@ __global__ void __launch_bounds__(kT, 1) k_tr_step(const __grid_constant__ StepA
   for (int ph = 0; go && ph < a.n_ph; ++ph) {
     const TrArgs& P = a.ph[ph];
     for (int b = blockIdx.x; b < P.n_cta; b += gridDim.x) {
-      tr_tile_pre(P, b, smem);
-      if (!tr_tile(P, b, smem, tmem, par, true, false)) {
+      tr_tile_pre<false>(P, b, smem, true);
+      if (!tr_tile<false>(P, b, smem, tmem, par, true, false)) {
         if (tid == 0) atomicExch(a.bar + 1, 1u);
         go = false;
         break;
@@ -901,7 +945,7 @@ __global__ void __launch_bounds__(kT, 1) k_tr_step(const __grid_constant__ StepA
 }
 
 int gemm_smem_bytes() {
-  return 1024 + kMaxChunks * (kM * 128 + 256 * 128) + 128 + (256 + 256 + 8 * 256 + 8 * 128 + 128 + 128 + 8) * 4;
+  return 1024 + kStageRegion + kTailBar + (256 + 256 + 8 * 256 + 8 * 128 + 128 + 128 + 8) * 4;
 }
 
 TrArgs tr_args(const Ctx& c, const TrJob& j0, const TrJob* j1, int* err) {
@@ -911,10 +955,12 @@ TrArgs tr_args(const Ctx& c, const TrJob& j0, const TrJob* j1, int* err) {
   a.drop_thr = c.cfg.dropout > 0.0f ? (uint64_t)std::ceil((double)c.cfg.dropout * 9007199254740992.0) : 0;
   a.drop_scale = (float)(1.0 / (1.0 - (double)c.cfg.dropout));
   a.job[0] = j0;
+  a.job[0].stages = tr_stages(j0.NT);
   a.n_cta0 = j0.m_tiles * j0.n_split * j0.splits;
   int n = a.n_cta0;
   if (j1) {
     a.job[1] = *j1;
+    a.job[1].stages = tr_stages(j1->NT);
     n += j1->m_tiles * j1->n_split * j1->splits;
   }
   a.err = err;
@@ -926,30 +972,52 @@ cudaError_t launch_tr_gemm(const Ctx& c, const TrJob& j0, const TrJob* j1, int* 
   const TrArgs a = tr_args(c, j0, j1, err);
   const int n = a.n_cta;
   const int smem = gemm_smem_bytes();
-  cudaError_t e = cudaFuncSetAttribute(k_tr_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  auto* k = c.tf.wide ? k_tr_gemm<true> : k_tr_gemm<false>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   // the column parts of a TE_FWD_OUT tile exchange row sums through
   // distributed shared memory: one cluster per tile
   const int cl = (j0.epi == TE_FWD_OUT && !j1) ? j0.n_split : 1;
-  return launch_chained(k_tr_gemm, dim3(n), dim3(kT), (size_t)smem, s, cl, a);
+  return launch_chained(k, dim3(n), dim3(kT), (size_t)smem, s, cl, a);
 }
 
-// Column parts per tile: two when the columns split into halves that are
-// multiples of 64 (each warp then owns a multiple of 16 columns).
-int n_split_for(int N) { return N % 128 == 0 ? 2 : 1; }
+// Column parts per tile of a product with N columns: two when the columns
+// split into halves that are multiples of 64 (each warp then owns a multiple
+// of 16 columns); wider layers, 128 columns a part (see plan_train_fast).
+int n_split_for(int N) { return N > 256 ? N / 128 : N % 128 == 0 ? 2 : 1; }
+
+// Column parts of a hidden forward product (per-launch path) over T row
+// tiles.  256 columns run as four 64-column parts (128 CTAs for a batch of
+// 4096: half the epilogue and image stores per SM); wider layers as 128-column
+// parts while those fill half the SMs, else 64-column ones.
+int n_split_fwd(int N, int T, int sms) {
+  if (N > 256) return T * (N / 128) >= sms / 2 ? N / 128 : N / 64;
+  return N % 256 == 0 ? 4 : n_split_for(N);
+}
+
+// Column parts of the last hidden layer's product, which form a cluster: two
+// halves, or four quarters of 512 columns (an accumulator has at most 256).
+int n_split_out(int N) { return N == 512 ? 4 : N > 256 ? 2 : n_split_for(N); }
 
 }  // namespace
 
 // The fast path applies to bf16 predictors with at least one hidden layer,
-// hidden widths that are multiples of 64 up to 256 and an input width of at
-// most 256 (padded to 64).
+// hidden widths that are multiples of 64 up to 256, or 384 or 512, and an
+// input width of at most 256 (padded to 64).  Layers wider than 256 stream
+// their K-blocks through the stages and split into parts of 128 columns; 320
+// and 448 have no such split into equal parts for the output product's
+// cluster of two or four and stay on the general path.  A step of
+// 128-512-512-1 at batch 4096 took 214 us on the general path (22 launches,
+// fp32 operands converted as they are staged) and takes 66 us here.
 bool plan_train_fast(const MlpDesc& m, int max_batch, TrainFast& f) {
   f = TrainFast{};
   if (!m.bf16 || m.n_layers < 2) return false;
   f.in_pad[0] = ((m.w[0] + 63) / 64) * 64;
   if (f.in_pad[0] > 256) return false;
   for (int l = 1; l < m.n_layers; ++l) {
-    if (m.w[l] % 64 != 0 || m.w[l] > 256) return false;
+    const bool wide = m.w[l] == 384 || m.w[l] == 512;
+    if (m.w[l] % 64 != 0 || (m.w[l] > 256 && !wide)) return false;
+    f.wide = f.wide || wide;
     f.in_pad[l] = m.w[l];
   }
   f.rows_max = ((max_batch + kM - 1) / kM) * kM;
@@ -1103,10 +1171,9 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
     J.epi = last ? TE_FWD_OUT : TE_FWD;
     J.m_tiles = T;
     // the persistent launch has no clusters: the output layer's row dot
-    // products stay within one CTA (all columns of the tile).  A hidden
-    // layer of 256 columns runs as four 64-column parts (128 CTAs for a
-    // batch of 4096: half the epilogue and image stores per SM)
-    J.n_split = (last && one) ? 1 : (!last && !one && m.w[l + 1] % 256 == 0) ? 4 : n_split_for(m.w[l + 1]);
+    // products stay within one CTA (all columns of the tile)
+    const int N = m.w[l + 1];
+    J.n_split = one ? (last ? 1 : n_split_for(N)) : last ? n_split_out(N) : n_split_fwd(N, T, c.sms);
     J.splits = 1;
     J.nchunks = J.kblocks = f.in_pad[l] / 64;
     J.NT = m.w[l + 1] / J.n_split;
@@ -1151,8 +1218,10 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
     W.m_tiles = (out + kM - 1) / kM;
     W.n_split = n_split_for(f.in_pad[l]);
     // K-blocks (of 64 batch rows) per CTA: 4 when that still gives 48 CTAs,
-    // else 2 (more CTAs, more partials for the optimiser to add)
-    const int kpc = W.m_tiles * W.n_split * (R / 256) >= 48 ? 4 : 2;
+    // else 2 (more CTAs, more partials for the optimiser to add); 8 where a
+    // wide layer's parts give 96 CTAs all the same (half the partials)
+    const int parts = W.m_tiles * W.n_split;
+    const int kpc = f.wide && parts * (R / 512) >= 96 ? 8 : parts * (R / 256) >= 48 ? 4 : 2;
     W.kblocks = R / 64;
     W.nchunks = std::min(kpc, W.kblocks);
     W.splits = (W.kblocks + W.nchunks - 1) / W.nchunks;  // the last one may be short

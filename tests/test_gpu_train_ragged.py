@@ -6,6 +6,7 @@ import torch
 
 from paper_2606_00946_gb300 import build as B
 from paper_2606_00946_gb300 import harness as H
+from paper_2606_00946_gb300 import lodestar as L
 
 pytestmark = pytest.mark.gpu
 
@@ -38,7 +39,11 @@ def reference_gradient(flat, widths, x, y):
 
 # batches whose 64-row blocks leave a short last split (and some that do not)
 @pytest.mark.parametrize("hidden,batch", [((256, 256), 3200), ((256, 256), 4096), ((256, 256, 256), 3900),
-                                          ((128, 128), 1), ((64,), 129), ((256, 256), 8100)])
+                                          ((128, 128), 1), ((64,), 129), ((256, 256), 8100),
+                                          # wider than 256: K-blocks streamed through the stages, parts of 128 (or,
+                                          # for few rows, 64) columns, clusters of two and four
+                                          ((512, 512), 4096), ((512, 512), 130), ((384, 384), 3200), ((128, 512), 700),
+                                          ((512, 64, 384), 1100), ((512,), 1), ((448, 512), 300)])
 def test_every_row_reaches_the_gradient(hidden, batch):
     d_inst, d_req = 34, 24
     widths = [6 + d_inst + d_req, *hidden, 1]
@@ -65,3 +70,8 @@ def test_every_row_reaches_the_gradient(hidden, batch):
     bound = 5e-3 * want.norm() + 2.0 ** -23 * flat.double().norm() / lr
     assert float((got - want).norm()) <= float(bound)
     r.close()
+
+
+def test_dropout_needs_hidden_widths_up_to_256():
+    with pytest.raises(L.LodestarError):
+        H.Router([64, 512, 512, 1], 34, 24, "bf16", dropout=0.1)
