@@ -316,8 +316,8 @@ int ls_read_features(ls_ctx *ctx, int64_t row0, int64_t n_rows, uint16_t *out, v
  * scores_opt / hits_opt (DEVICE [n_req, n_inst], nullable): each request's
  * predictions and hit lengths as seen when it was decided.  Needs the prefix
  * index mode and n_inst x (widest layer) small enough for one CTA's shared
- * memory (LS_ERR_ARG otherwise; the large cluster is beyond it).  One CTA walks
- * the requests, so the call's time grows with n_req.  Other arguments, the
+ * memory (LS_ERR_ARG otherwise; the large cluster is beyond it).  One cluster of
+ * CTAs walks the requests, so the call's time grows with n_req.  Other arguments, the
  * stream rules and errors are those of ls_route_batch. */
 int ls_route_sequential(ls_ctx *ctx, int32_t n_req, const int32_t *tok, const int64_t *tok_off,
                         const float *req_feats, int32_t queue_col, int32_t *choice, float *best, float *scores_opt,
