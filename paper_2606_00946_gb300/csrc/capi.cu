@@ -277,7 +277,11 @@ int ls_create(const ls_config* cfg, ls_ctx** out) {
   A(dalloc(&c.dz1, B * m.max_width));
   A(dalloc(&c.grad, c.n_params));
   c.gpart_floats = 64 * max_wl + 64 * (int64_t)m.max_width;  // dW partials, then column-sum partials
+  int64_t trs_floats = 0;  // the fp32 step takes its partials' space here (it uses none of the general step's)
+  const bool trs = plan_train_f32(m, c.n_params, cfg->max_train_batch, c.sms, &trs_floats);
+  c.gpart_floats = std::max(c.gpart_floats, trs_floats);
   A(dalloc(&c.gpart, c.gpart_floats));
+  if (trs) c.trs_part = c.gpart;
   A(dalloc(&c.loss_tmp, 1));
   A(dalloc(&c.d_err, 1));
   A(dalloc(&c.st, 1));
@@ -799,8 +803,9 @@ int ls_train_step(ls_ctx* h, int32_t batch, const int32_t* idx, int32_t opt, flo
   if (!c.have_params) return fail(LS_ERR_STATE, "parameters not set");
   if (!c.have_norm) return fail(LS_ERR_STATE, "normaliser not set");
   if (c.ring_enqueued < 1) return fail(LS_ERR_STATE, "sample ring is empty");
-  LS_CK(c.tf.on ? run_train_fast(c, batch, idx, opt, lr, loss_out, S(stream))
-                : run_train_step(c, batch, idx, opt, lr, loss_out, S(stream)));
+  LS_CK(c.tf.on      ? run_train_fast(c, batch, idx, opt, lr, loss_out, S(stream))
+        : c.trs_part ? run_train_f32(c, batch, idx, opt, lr, loss_out, S(stream))
+                     : run_train_step(c, batch, idx, opt, lr, loss_out, S(stream)));
   return LS_OK;
 }
 

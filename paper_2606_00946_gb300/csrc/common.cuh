@@ -274,6 +274,7 @@ struct Ctx {
   int64_t gpart_floats = 0;
   float* loss_tmp = nullptr;  // [1]
   TrainFast tf;               // tensor-core training buffers (when tf.on)
+  float* trs_part = nullptr;  // fp32 step (k_train_f32.cu): gradient partials per CTA, in gpart (null: not used)
   int train_ctas = 0;         // > 0: persistent training step of that many CTAs
   uint32_t* tr_bar = nullptr; // [2]: its grid-barrier arrivals and abort flag
 
@@ -511,6 +512,9 @@ void train_fast_bind(const MlpDesc& m, TrainFast& f, uint8_t* base, float* parts
 cudaError_t train_fast_images(Ctx& c, cudaStream_t s);
 cudaError_t run_train_fast(Ctx& c, int batch, const int32_t* idx, int opt, float lr, float* loss_out,
                            cudaStream_t s);
+bool plan_train_f32(const MlpDesc& m, int64_t n_params, int max_batch, int sms, int64_t* part_floats);
+cudaError_t run_train_f32(Ctx& c, int batch, const int32_t* idx, int opt, float lr, float* loss_out,
+                          cudaStream_t s);
 void set_last_error(const char* msg);  // sets the text ls_last_error() returns
 cudaError_t launch_prefix_index(int n_req, const int32_t* tok, const int64_t* tok_off, const uint64_t* gkeys,
                                 const uint64_t* gmask, int W, uint64_t gmask_slots, int n_inst, int32_t* hits,

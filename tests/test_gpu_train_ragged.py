@@ -16,9 +16,9 @@ def _built():
     B.build()
 
 
-def reference_gradient(flat, widths, x, y):
-    """Gradient of the minibatch loss with the products' operands in bf16, sums in fp64."""
-    r = lambda t: t.float().bfloat16().double()
+def reference_gradient(flat, widths, x, y, bf16=True):
+    """Gradient of the minibatch loss (the products' operands in bf16 where asked), sums in fp64."""
+    r = lambda t: t.float().bfloat16().double() if bf16 else t.double()
     layers, o = [], 0
     for a, b in zip(widths[:-1], widths[1:]):
         layers.append((flat[o:o + a * b].view(b, a).double(), flat[o + a * b:o + a * b + b].double()))
@@ -69,6 +69,47 @@ def test_every_row_reaches_the_gradient(hidden, batch):
     # and the fp32 subtraction of the update (2^-24 |p| / lr)
     bound = 5e-3 * want.norm() + 2.0 ** -23 * flat.double().norm() / lr
     assert float((got - want).norm()) <= float(bound)
+    r.close()
+
+
+# fp32 tiles of 4, 8, 16 and 32 rows, several tiles per CTA, odd widths,
+# weights resident and staged in chunks, no hidden layer
+@pytest.mark.parametrize("hidden,batch", [((64, 64), 1), ((64, 64), 256), ((64, 64), 700), ((64, 64), 1300),
+                                          ((64, 64), 3001), ((64, 64), 6000), ((100, 50), 333), ((33, 7, 65), 130),
+                                          ((128, 128, 128), 1024), ((256, 256), 515), ((1000,), 90), ((), 257),
+                                          ((300, 200, 100), 64)])
+def test_every_row_reaches_the_fp32_gradient(hidden, batch):
+    d_inst, d_req = 34, 24
+    widths = [6 + d_inst + d_req, *hidden, 1]
+    ring = batch + 37
+    r = H.Router(widths, d_inst, d_req, "f32", max_instances=4, max_requests=4, max_keys_per_instance=64,
+                 ring_capacity=ring, max_train_batch=batch, max_batch_tokens=64)
+    g = torch.Generator(device="cuda").manual_seed(batch)
+    x = torch.randn(ring, widths[0], generator=g, device="cuda")
+    y = torch.randn(ring, generator=g, device="cuda")
+    flat = torch.cat([torch.cat([torch.randn(b * a, generator=g, device="cuda") / a ** 0.5,
+                                 torch.randn(b, generator=g, device="cuda") * 0.1])
+                      for a, b in zip(widths[:-1], widths[1:])])
+    idx = torch.randperm(ring, generator=g, device="cuda")[:batch].int()
+    y[idx[-1]] += 50.0  # the last row carries much of the gradient
+    r.set_normalizer(torch.zeros(widths[0], device="cuda"), torch.ones(widths[0], device="cuda"))
+    r.set_params(flat)
+    r.log(x, y)
+    lr, loss = 1e-2, torch.zeros(1, device="cuda")
+    r.train(batch, idx, opt="sgd", lr=lr, loss_out=loss)
+    got = (flat.double() - r.get_params().double()) / lr
+    assert r.sync() == 0
+    xi, yi = x[idx.long()], y[idx.long()]
+    want = reference_gradient(flat, widths, xi, yi, bf16=False)
+    # fp32 sums of up to `batch` terms (2^-24 sqrt(n) of the norm, a few layers deep; a ReLU whose input lies within
+    # rounding of 0 may go the other way for a row) and the update's fp32 subtraction
+    bound = 2e-5 * want.norm() + 2.0 ** -23 * flat.double().norm() / lr
+    assert float((got - want).norm()) <= float(bound)
+    # twice the same step from the same state: the same bits
+    p1 = r.get_params()
+    r.set_params(flat)
+    r.train(batch, idx, opt="sgd", lr=lr, loss_out=loss)
+    assert torch.equal(p1, r.get_params())
     r.close()
 
 
