@@ -117,7 +117,7 @@ void free_all(Ctx& c) {
                   c.gpart, c.loss_tmp, c.d_err, c.pub[0].img, c.pub[1].img, c.xin, c.xrq, c.pairx, c.ximg,
                   c.bkeys, c.work, c.work_n, c.gkeys, c.gmask, c.st, c.tf.base, c.tf.parts,
                   c.pub[0].bounds, c.pub[1].bounds, c.bounds_stage, c.benc, c.remb, c.rnorm, c.rpart, c.rd,
-                  c.rn, c.rinv, c.rcount, c.rimg, c.rrank, c.tr_bar};
+                  c.rn, c.rinv, c.rcount, c.rimg, c.rrank, c.tr_bar, c.trs_part};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c.ev_pub) cudaEventDestroy(c.ev_pub);
@@ -270,23 +270,29 @@ int ls_create(const ls_config* cfg, ls_ctx** out) {
   }
   A(dalloc(&c.hits, R * NI));
   A(dalloc(&c.scores, R * NI));
-  A(dalloc(&c.tx, B * sum_in));
-  A(dalloc(&c.tz, B * sum_out));
+  // training scratch: what the context's path uses (k_train_fast.cu,
+  // k_train_f32.cu, else the general step of k_train.cu)
+  const bool fast_train = plan_train_fast(m, cfg->max_train_batch, c.tf);
+  int64_t trs_floats = 0;
+  const bool trs = !fast_train && plan_train_f32(m, c.n_params, cfg->max_train_batch, c.sms, &trs_floats);
+  const bool general = !fast_train && !trs;
+  if (general || cfg->replay_capacity > 0) {  // (replay admission runs the general forward)
+    A(dalloc(&c.tx, B * sum_in));
+    A(dalloc(&c.tz, B * sum_out));
+  }
   A(dalloc(&c.ty, B));
-  A(dalloc(&c.dz0, B * m.max_width));
-  A(dalloc(&c.dz1, B * m.max_width));
-  A(dalloc(&c.grad, c.n_params));
-  c.gpart_floats = 64 * max_wl + 64 * (int64_t)m.max_width;  // dW partials, then column-sum partials
-  int64_t trs_floats = 0;  // the fp32 step takes its partials' space here (it uses none of the general step's)
-  const bool trs = plan_train_f32(m, c.n_params, cfg->max_train_batch, c.sms, &trs_floats);
-  c.gpart_floats = std::max(c.gpart_floats, trs_floats);
-  A(dalloc(&c.gpart, c.gpart_floats));
-  if (trs) c.trs_part = c.gpart;
+  if (general) {
+    A(dalloc(&c.dz0, B * m.max_width));
+    A(dalloc(&c.dz1, B * m.max_width));
+    A(dalloc(&c.grad, c.n_params));
+    c.gpart_floats = 64 * max_wl + 64 * (int64_t)m.max_width;  // dW partials, then column-sum partials
+    A(dalloc(&c.gpart, c.gpart_floats));
+  }
+  if (trs) A(dalloc(&c.trs_part, trs_floats));
   A(dalloc(&c.loss_tmp, 1));
   A(dalloc(&c.d_err, 1));
   A(dalloc(&c.st, 1));
   int64_t tf_bytes = 0;
-  const bool fast_train = plan_train_fast(m, cfg->max_train_batch, c.tf);
   if (cfg->dropout > 0.0f && (!fast_train || c.tf.wide)) {
     free_all(c);
     delete h;
@@ -564,7 +570,8 @@ int route_impl(ls_ctx* h, int32_t n_req, const int32_t* tok, const int64_t* tok_
   if (weight_version_out) *weight_version_out = v;
   if (n_req == 0) return LS_OK;
   int32_t* hits = hits_opt ? hits_opt : c.hits;
-  const bool fused_select = !guarded && c.use_tc && scorer_selects(c.tc, c.n_inst);
+  const bool fused_select = !guarded && (c.use_tc ? scorer_selects(c.tc, c.n_inst)
+                                                  : simt_selects(c.mlp, n_req, c.n_inst, c.sms));
   float* scores = scores_opt ? scores_opt : (fused_select ? nullptr : c.scores);
   if (c.use_index) {
     LS_CK(traced(c, TR_PREFIX_INDEX, 1, s, [&] {
@@ -604,7 +611,8 @@ int route_impl(ls_ctx* h, int32_t n_req, const int32_t* tok, const int64_t* tok_
   } else {
     LS_CK(traced(c, TR_SCORE, 1, s, [&] {
       return launch_score_simt(c.mlp, c.pub, &c.st->route_b, n_req, c.n_inst, tok_off, hits, c.inst_state,
-                               c.cfg.d_inst, req_feats, c.cfg.d_req, c.mean, c.stdv, scores, s);
+                               c.cfg.d_inst, req_feats, c.cfg.d_req, c.mean, c.stdv, scores,
+                               fused_select ? choice : nullptr, fused_select ? best : nullptr, c.sms, s);
     }));
   }
   if (guarded)

@@ -263,7 +263,7 @@ struct Ctx {
   bool use_tc = false;
   TcPlan tc;
 
-  // train scratch
+  // train scratch (what the context's training path does not use is null)
   float* tx = nullptr;        // activations a_0..a_{L-1}, [B, sum w[0..L-1]]
   float* tz = nullptr;        // pre-activations z_1..z_L, [B, sum w[1..L]]
   float* ty = nullptr;        // targets [B]
@@ -274,7 +274,7 @@ struct Ctx {
   int64_t gpart_floats = 0;
   float* loss_tmp = nullptr;  // [1]
   TrainFast tf;               // tensor-core training buffers (when tf.on)
-  float* trs_part = nullptr;  // fp32 step (k_train_f32.cu): gradient partials per CTA, in gpart (null: not used)
+  float* trs_part = nullptr;  // fp32 step (k_train_f32.cu): gradient partials per CTA (null: not used)
   int train_ctas = 0;         // > 0: persistent training step of that many CTAs
   uint32_t* tr_bar = nullptr; // [2]: its grid-barrier arrivals and abort flag
 
@@ -428,7 +428,11 @@ cudaError_t launch_assemble_features(int n_req, int n_inst, const int64_t* tok_o
 cudaError_t launch_score_simt(const MlpDesc& mlp, const Published* pub, const int32_t* sel, int n_req, int n_inst,
                               const int64_t* tok_off, const int32_t* hits, const float* inst_state,
                               int d_inst, const float* req_feats, int d_req, const float* mean,
-                              const float* stdv, float* scores, cudaStream_t s);
+                              const float* stdv, float* scores, int32_t* choice, float* best, int sms,
+                              cudaStream_t s);
+// Whether the CUDA-core scorer runs the selector for this batch (choice and
+// best non-NULL; scores then only when non-NULL).
+bool simt_selects(const MlpDesc& m, int n_req, int n_inst, int sms);
 cudaError_t launch_argmin(int n_req, int n_inst, const float* scores, int32_t* choice,
                           float* best, cudaStream_t s);
 // Algorithm 4 guards.  benc must hold the identity codes (0xff800000 in
