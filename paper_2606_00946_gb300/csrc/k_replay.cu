@@ -167,6 +167,8 @@ __global__ void k_rowmin_reduce(int M, int parts, const float* __restrict__ part
 // Both pools' partial minima (rows [0, P) candidates, [P, P + Rc) kept).
 __global__ void k_rowmin_reduce2(int P, int rows, int parts, const float* __restrict__ part, int64_t ldp,
                                  float* __restrict__ dc, float* __restrict__ nk) {
+  pdl_wait();
+  pdl_trigger();
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < rows; r += (int64_t)gridDim.x * blockDim.x) {
     float best = INFINITY;
     for (int q = 0; q < parts; ++q) best = fminf(best, part[r * ldp + q]);
@@ -182,13 +184,19 @@ __device__ __forceinline__ float div_key(float v) { return isnan(v) ? -INFINITY 
 // ---------------------------------------------------------------------------
 // The image holds the embeddings as 128-row tiles (candidate tiles, then kept
 // tiles) of H/64 K-major 128-byte-swizzled slabs of 16 KB, so one bulk copy
-// per slab lands a tile in the MMA layout.  CTA (row tile, column split):
+// lands a tile in the MMA layout.  CTA (row tile, column split):
 // its 128 rows against a range of kept 128-row column tiles; warp 0 issues
 // the MMAs into two TMEM accumulators, warp 1 bulk-copies the row tile once
-// and the column tiles through two buffers, warps 2..5 (one TMEM lane
-// quadrant each) turn each accumulator into the row minima of
-// |g_r|^2 + |g_c|^2 - 2 g_r.g_c (the row's own kept column skipped).
-constexpr int kDistThreads = 192;
+// and the column tiles through two buffers, warps 2..9 (two per TMEM lane
+// quadrant, a column half each) turn each accumulator into the row minima of
+// |g_r|^2 + |g_c|^2 - 2 g_r.g_c (the row's own kept column skipped).  A warp
+// loads its 64 column norms of a tile ahead, two a lane, and reads them back
+// from shared memory four at a time; only the tile that holds the rows' own
+// columns looks for them.  (Four epilogue warps with a global load per column
+// and row left the products waiting.  With this, the ranks by tiles of one
+// comparison and the chained launches, an admission round of 1000 candidates
+// against pools of 5000 x 128 took 160 us, from 213.)
+constexpr int kDistThreads = 320;
 constexpr int kSlab = 16384;       // 128 rows x 64 bf16
 
 struct DistArgs {
@@ -207,8 +215,9 @@ __global__ void __launch_bounds__(kDistThreads, 1) k_dist_rowmin(const __grid_co
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int kb = a.H / 64;
   uint8_t* sA = smem;
-  uint8_t* sB[2] = {smem + kb * kSlab, smem + 2 * kb * kSlab};
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + 3 * kb * kSlab);
+  uint8_t *sB0 = smem + kb * kSlab, *sB1 = smem + 2 * kb * kSlab;
+  float* s_nb = reinterpret_cast<float*>(smem + 3 * kb * kSlab);  // [8][64] column norms by epilogue warp
+  uint64_t* bar = reinterpret_cast<uint64_t*>(s_nb + 8 * 64);
   uint64_t *a_full = bar, *b_full = bar + 1, *b_empty = bar + 3, *acc_full = bar + 5, *acc_empty = bar + 7;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bar + 9);
 
@@ -216,18 +225,20 @@ __global__ void __launch_bounds__(kDistThreads, 1) k_dist_rowmin(const __grid_co
   const int tile = blockIdx.x / a.splits, split = blockIdx.x - tile * a.splits;
   const bool kept_rows = tile >= a.tilesC;
   const int rtile = kept_rows ? tile - a.tilesC : tile;       // row tile inside its region
+  pdl_wait();
+  pdl_trigger();
   const int64_t rows_used = kept_rows ? a.counts[1] : a.counts[0];
   const int64_t ktiles_used = (a.counts[1] + 127) / 128;
   const int t0 = split * a.per_split;
   int T = (int)(ktiles_used - t0);
   T = T < 0 ? 0 : (T > a.per_split ? a.per_split : T);
   const int base_row = kept_rows ? a.P : 0;                   // first norm / partial row of the region
-  // epilogue thread -> row: warps 2..5 own TMEM lane quadrants warp & 3
-  const int q = warp & 3;
+  // epilogue thread -> row: warps 2..9 own TMEM lane quadrants warp & 3, and a column half each
+  const int q = warp & 3, half = warp >= 6 ? 1 : 0;
   const int row = rtile * 128 + 32 * q + lane;                // row inside the region
   const int region_rows = kept_rows ? a.Rc : a.P;
   if ((int64_t)rtile * 128 >= rows_used || T == 0) {          // nothing of this CTA is in use
-    if (warp >= 2 && row < region_rows) a.part[(int64_t)(base_row + row) * a.ldp + split] = INFINITY;
+    if (warp >= 2 && row < region_rows) a.part[(int64_t)(base_row + row) * a.ldp + 2 * split + half] = INFINITY;
     return;
   }
   if (tid == 0) {
@@ -236,7 +247,7 @@ __global__ void __launch_bounds__(kDistThreads, 1) k_dist_rowmin(const __grid_co
       mbar_init(b_full + i, 1);
       mbar_init(b_empty + i, 1);
       mbar_init(acc_full + i, 1);
-      mbar_init(acc_empty + i, 4);
+      mbar_init(acc_empty + i, 8);
     }
     fence_mbar_init();
   }
@@ -256,14 +267,13 @@ __global__ void __launch_bounds__(kDistThreads, 1) k_dist_rowmin(const __grid_co
   if (warp == 1) {
     if (lane == 0) {
       mbar_arrive_expect_tx(a_full, tile_bytes);
-      for (int k = 0; k < kb; ++k) bulk_g2s(sA + k * kSlab, imgA + k * kSlab, kSlab, a_full);
+      bulk_g2s(sA, imgA, tile_bytes, a_full);
       for (int t = 0; t < T && ok; ++t) {
         const int b = t & 1;
         if (t >= 2 && !mbar_wait(b_empty + b, (uint32_t)(((t - 2) >> 1) & 1))) ok = false;
         if (!ok) break;
         mbar_arrive_expect_tx(b_full + b, tile_bytes);
-        for (int k = 0; k < kb; ++k)
-          bulk_g2s(sB[b] + k * kSlab, imgB + (int64_t)t * tile_bytes + k * kSlab, kSlab, b_full + b);
+        bulk_g2s(b ? sB1 : sB0, imgB + (int64_t)t * tile_bytes, tile_bytes, b_full + b);
       }
       if (!ok) latch_error(a.err, LS_ERR_TIMEOUT);
     }
@@ -276,7 +286,7 @@ __global__ void __launch_bounds__(kDistThreads, 1) k_dist_rowmin(const __grid_co
         if (!mbar_wait(b_full + b, (uint32_t)((t >> 1) & 1))) { ok = false; break; }
         if (t >= 2 && !mbar_wait(acc_empty + b, (uint32_t)(((t - 2) >> 1) & 1))) { ok = false; break; }
         tc_fence_after();
-        const uint32_t ab = smem_u32(sA), bb = smem_u32(sB[b]);
+        const uint32_t ab = smem_u32(sA), bb = smem_u32(b ? sB1 : sB0);
         for (int k = 0; k < kb; ++k)
 #pragma unroll
           for (int j = 0; j < 4; ++j)
@@ -289,67 +299,106 @@ __global__ void __launch_bounds__(kDistThreads, 1) k_dist_rowmin(const __grid_co
     }
   } else {
     const float na = row < region_rows ? __ldg(a.norm + base_row + row) : INFINITY;
-    const int self = kept_rows ? row : -1;                    // the row's own kept column
     const uint32_t lane_addr = (uint32_t)(32 * q) << 16;
     float rmin = INFINITY;
+    float* nbw = s_nb + 64 * (warp - 2);
+    const auto norm_at = [&](int t, int u) {  // this lane's column lane + 32 u of the warp's half of tile t
+      const int col = (t0 + t) * 128 + 64 * half + 32 * u + lane;
+      return t < T && col < a.Rc ? __ldg(a.norm + a.P + col) : INFINITY;
+    };
+    float n0 = norm_at(0, 0), n1 = norm_at(0, 1);
     for (int t = 0; t < T; ++t) {
       const int b = t & 1;
-      const int col0 = (t0 + t) * 128;
+      __syncwarp();  // the tile before is read
+      nbw[lane] = n0;
+      nbw[32 + lane] = n1;
+      __syncwarp();
+      n0 = norm_at(t + 1, 0);
+      n1 = norm_at(t + 1, 1);
       if (!mbar_wait(acc_full + b, (uint32_t)((t >> 1) & 1))) {
         if (lane == 0) latch_error(a.err, LS_ERR_TIMEOUT);
         break;
       }
       tc_fence_after();
-      for (int c = 0; c < 128; c += 32) {
-        float nb[32];
-#pragma unroll
-        for (int u = 0; u < 32; ++u) nb[u] = col0 + c + u < a.Rc ? __ldg(a.norm + a.P + col0 + c + u) : INFINITY;
+      // the column of this tile that is the row itself (-1: none)
+      const int self = kept_rows && t0 + t == rtile ? 32 * q + lane : -1;
+      const bool diag = kept_rows && t0 + t == rtile;
+#pragma unroll 1
+      for (int c = 64 * half; c < 64 * half + 64; c += 32) {
         uint32_t v[32];
         tmem_ld32(tmem + lane_addr + (uint32_t)(128 * b + c), v);
         tmem_wait_ld();
+        const float4* nb4 = reinterpret_cast<const float4*>(nbw + (c & 32));
 #pragma unroll
-        for (int u = 0; u < 32; ++u) {
-          const float dist = na + nb[u] - 2.0f * __uint_as_float(v[u]);
-          if (col0 + c + u != self) rmin = fminf(rmin, dist);
+        for (int u4 = 0; u4 < 8; ++u4) {
+          const float4 n4 = nb4[u4];
+          const float nb[4] = {n4.x, n4.y, n4.z, n4.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int u = 4 * u4 + e;
+            const float dist = na + nb[e] - 2.0f * __uint_as_float(v[u]);
+            if (!diag || c + u != self) rmin = fminf(rmin, dist);
+          }
         }
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(acc_empty + b);
     }
-    if (row < region_rows) a.part[(int64_t)(base_row + row) * a.ldp + split] = rmin;
+    if (row < region_rows) a.part[(int64_t)(base_row + row) * a.ldp + 2 * split + half] = rmin;
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, 256);
 }
 
-// Ranks by counting, tiled over (element tile, key tile): each block counts,
-// for its 256 elements, the keys of one 1024-key tile that come before them
-// (candidates: larger d first; kept records: smaller n first; equal keys by
-// index) and adds the count to rank[] (integer sums: the order of the
-// additions does not matter).  rank[] was zeroed by k_replay_prep.
-__global__ void __launch_bounds__(256) k_replay_rank(ReplayGeom g, const int64_t* __restrict__ counts,
-                                                     const float* __restrict__ dc, const float* __restrict__ nk,
-                                                     int32_t* __restrict__ rank) {
-  __shared__ float tile[1024];
-  const int64_t cb = (g.P + 255) / 256;               // element tiles of the candidates
-  const bool cand = blockIdx.x < cb;
-  const int64_t i = (cand ? blockIdx.x : blockIdx.x - cb) * 256 + threadIdx.x;
+// Ranks by counting, tiled over (element tile, key tile) of kRankTile each:
+// each block counts, for its elements, the keys of one key tile that come
+// before them (candidates: larger d first; kept records: smaller n first;
+// equal keys by index) and adds the count to rank[] (integer sums: the order
+// of the additions does not matter).  rank[] was zeroed by k_replay_prep.
+// Off the diagonal every key of the tile has a lower, or every one a higher,
+// index than every element, so the tie rule is the comparison's strictness:
+// one comparison a pair.  (1024-key tiles with both comparisons in every pair:
+// 35 us for pools of 5000, 8 us now.)
+constexpr int kRankTile = 256;
+
+__global__ void __launch_bounds__(kRankTile) k_replay_rank(ReplayGeom g, const int64_t* __restrict__ counts,
+                                                           const float* __restrict__ dc,
+                                                           const float* __restrict__ nk, int32_t* __restrict__ rank) {
+  __shared__ __align__(16) float tile[kRankTile];
+  pdl_wait();
+  pdl_trigger();
+  const int cb = (int)((g.P + kRankTile - 1) / kRankTile);  // element tiles of the candidates
+  const bool cand = (int)blockIdx.x < cb;
+  const int et = cand ? blockIdx.x : blockIdx.x - cb, kt = blockIdx.y;
   const int64_t cnt = cand ? counts[0] : counts[1];
-  const int64_t base = (int64_t)blockIdx.y * 1024;
-  if ((cand ? blockIdx.x : blockIdx.x - cb) * 256 >= cnt || base >= cnt) return;   // block-uniform
+  const int64_t i = (int64_t)et * kRankTile + threadIdx.x, base = (int64_t)kt * kRankTile;
+  if ((int64_t)et * kRankTile >= cnt || base >= cnt) return;  // block-uniform
   const float* keys = cand ? dc : nk;
-  for (int q = threadIdx.x; q < 1024; q += 256) tile[q] = base + q < cnt ? div_key(keys[base + q]) : 0.0f;
+  // ascending order of v: d negated, so that larger d comes first (-inf, the
+  // key of NaN, last)
+  const float sign = cand ? -1.0f : 1.0f;
+  const float none = __int_as_float(0x7fc00000);  // past the records: before nothing
+  tile[threadIdx.x] = base + threadIdx.x < cnt ? sign * div_key(keys[base + threadIdx.x]) : none;
   __syncthreads();
   if (i >= cnt) return;
-  const float mine = div_key(keys[i]);
-  const int lim = cnt - base < 1024 ? (int)(cnt - base) : 1024;
+  const float mine = sign * div_key(keys[i]);
   int r = 0;
-  for (int q = 0; q < lim; ++q) {
-    const float o = tile[q];
-    const int64_t f = base + q;
-    r += cand ? (o > mine || (o == mine && f < i)) : (o < mine || (o == mine && f < i));
+  if (kt < et) {  // lower indices: equal keys come first
+#pragma unroll 8
+    for (int q = 0; q < kRankTile; q += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(tile + q);
+      r += (v.x <= mine) + (v.y <= mine) + (v.z <= mine) + (v.w <= mine);
+    }
+  } else if (kt > et) {
+#pragma unroll 8
+    for (int q = 0; q < kRankTile; q += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(tile + q);
+      r += (v.x < mine) + (v.y < mine) + (v.z < mine) + (v.w < mine);
+    }
+  } else {
+    for (int q = 0; q < kRankTile; ++q) r += tile[q] < mine || (tile[q] == mine && q < (int)threadIdx.x);
   }
   if (r) atomicAdd(rank + (cand ? 0 : g.P) + i, r);
 }
@@ -357,6 +406,8 @@ __global__ void __launch_bounds__(256) k_replay_rank(ReplayGeom g, const int64_t
 // inv[rank] = element (candidates at [0, P), kept records at [P, P + Rc)).
 __global__ void k_replay_inv(ReplayGeom g, const int64_t* __restrict__ counts, const int32_t* __restrict__ rank,
                              int32_t* __restrict__ inv) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t m = counts[0], nr = counts[1];
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < g.P + g.Rc;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -370,6 +421,8 @@ __global__ void k_replay_inv(ReplayGeom g, const int64_t* __restrict__ counts, c
 __global__ void __launch_bounds__(256) k_replay_apply(int d, ReplayGeom g, DevState* st, const float* __restrict__ dc,
                                                       const float* __restrict__ nk, const int32_t* __restrict__ inv,
                                                       float* ring_x, float* ring_y) {
+  pdl_wait();
+  pdl_trigger();
   int64_t lo, hi;
   pending_range(st, g, lo, hi);
   const int64_t m = hi - lo;
@@ -457,21 +510,20 @@ cudaError_t run_replay_admit(Ctx& c, float* d_out, float* n_out, cudaStream_t s)
     da.H = H;
     da.tilesC = tilesC;
     da.tilesK = tilesK;
-    da.splits = std::max(1, std::min(std::min(tilesK, kRowMinParts), 2 * c.sms / (tilesC + tilesK)));
+    da.splits = std::max(1, std::min(std::min(tilesK, kRowMinParts / 2), 2 * c.sms / (tilesC + tilesK)));
     da.per_split = (tilesK + da.splits - 1) / da.splits;
     da.err = c.d_err;
-    const int smem = 1024 + 3 * (H / 64) * kSlab + 128;
+    const int smem = 1024 + 3 * (H / 64) * kSlab + 8 * 64 * 4 + 128;
     e = traced(c, TR_REPLAY, 1, s, [&] {
       cudaError_t a = cudaFuncSetAttribute(k_dist_rowmin, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
       if (a != cudaSuccess) return a;
-      k_dist_rowmin<<<(tilesC + tilesK) * da.splits, kDistThreads, smem, s>>>(da);
-      return cudaGetLastError();
+      return launch_chained(k_dist_rowmin, dim3((tilesC + tilesK) * da.splits), dim3(kDistThreads), (size_t)smem, s, 1,
+                            da);
     });
     if (e != cudaSuccess) return e;
     e = traced(c, TR_REPLAY, 1, s, [&] {
-      k_rowmin_reduce2<<<grid_for(rows, c.sms), 256, 0, s>>>((int)g.P, (int)rows, da.splits, c.rpart, kRowMinParts,
-                                                             c.rd, c.rn);
-      return cudaGetLastError();
+      return launch_chained(k_rowmin_reduce2, dim3(grid_for(rows, c.sms)), dim3(256), 0, s, 1, (int)g.P, (int)rows,
+                            2 * da.splits, c.rpart, kRowMinParts, c.rd, c.rn);
     });
     if (e != cudaSuccess) return e;
   }
@@ -516,21 +568,22 @@ cudaError_t run_replay_admit(Ctx& c, float* d_out, float* n_out, cudaStream_t s)
   }
   // 3. ranks, 4. admission
   e = traced(c, TR_REPLAY, 1, s, [&] {
-    const dim3 grid((unsigned)((g.P + 255) / 256 + (g.Rc + 255) / 256),
-                    (unsigned)((std::max(g.P, g.Rc) + 1023) / 1024));
-    k_replay_rank<<<grid, 256, 0, s>>>(g, c.rcount, c.rd, c.rn, c.rrank);
-    return cudaGetLastError();
+    const unsigned kt = (unsigned)((std::max(g.P, g.Rc) + kRankTile - 1) / kRankTile);
+    const dim3 grid((unsigned)((g.P + kRankTile - 1) / kRankTile + (g.Rc + kRankTile - 1) / kRankTile), kt);
+    return launch_chained(k_replay_rank, grid, dim3(kRankTile), 0, s, 1, g, c.rcount, c.rd, c.rn, c.rrank);
   });
   if (e != cudaSuccess) return e;
   e = traced(c, TR_REPLAY, 1, s, [&] {
-    k_replay_inv<<<grid_for(g.P + g.Rc, c.sms), 256, 0, s>>>(g, c.rcount, c.rrank, c.rinv);
-    return cudaGetLastError();
+    return launch_chained(k_replay_inv, dim3(grid_for(g.P + g.Rc, c.sms)), dim3(256), 0, s, 1, g, c.rcount, c.rrank,
+                          c.rinv);
   });
   if (e != cudaSuccess) return e;
   return traced(c, TR_REPLAY, 1, s, [&] {
-    k_replay_apply<<<grid_for(g.P * 32, c.sms), 256, 0, s>>>(m.w[0], g, c.st, c.rd, c.rn, c.rinv, c.ring_x,
-                                                             c.ring_y);
-    return cudaGetLastError();
+    // a block per SM at most: each arrives once at the counter the last one
+    // resets (625 arrivals took most of 12 us)
+    const int blocks = (int)std::min<int64_t>((g.P + 7) / 8, c.sms);
+    return launch_chained(k_replay_apply, dim3(blocks), dim3(256), 0, s, 1, m.w[0], g, c.st, c.rd, c.rn, c.rinv,
+                          c.ring_x, c.ring_y);
   });
 }
 
