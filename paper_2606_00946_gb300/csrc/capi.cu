@@ -117,7 +117,7 @@ void free_all(Ctx& c) {
                   c.gpart, c.loss_tmp, c.d_err, c.pub[0].img, c.pub[1].img, c.xin, c.xrq, c.pairx, c.ximg,
                   c.bkeys, c.work, c.work_n, c.gkeys, c.gmask, c.st, c.tf.base, c.tf.parts,
                   c.pub[0].bounds, c.pub[1].bounds, c.bounds_stage, c.benc, c.remb, c.rnorm, c.rpart, c.rd,
-                  c.rn, c.rinv, c.rcount, c.rimg, c.rrank, c.tr_bar, c.trs_part};
+                  c.rn, c.rinv, c.rcount, c.rimg, c.rrank, c.tr_bar, c.trs_part, c.remb_img};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c.ev_pub) cudaEventDestroy(c.ev_pub);
@@ -276,7 +276,13 @@ int ls_create(const ls_config* cfg, ls_ctx** out) {
   int64_t trs_floats = 0;
   const bool trs = !fast_train && plan_train_f32(m, c.n_params, cfg->max_train_batch, c.sms, &trs_floats);
   const bool general = !fast_train && !trs;
-  if (general || cfg->replay_capacity > 0) {  // (replay admission runs the general forward)
+  // replay admission embeds its records on the fast path's images, or through the general forward
+  if (cfg->replay_capacity > 0 && c.rimg) {
+    const int64_t tiles = (cfg->pending_capacity + 127) / 128 + (cfg->replay_capacity + 127) / 128;
+    const int64_t bytes = replay_embed_bytes(m, c.tf, 128 * tiles);
+    if (bytes) A(dalloc(&c.remb_img, bytes));
+  }
+  if (general || (cfg->replay_capacity > 0 && !c.remb_img)) {
     A(dalloc(&c.tx, B * sum_in));
     A(dalloc(&c.tz, B * sum_out));
   }

@@ -236,6 +236,7 @@ struct Ctx {
   int32_t* rrank = nullptr;       // rank of each candidate [P], then of each kept record [Rc]
   int64_t* rcount = nullptr;      // candidates and kept records of the round in flight [2]
   uint8_t* rimg = nullptr;        // bf16 embedding image (128-row tiles, MMA layout) for bf16 predictors
+  uint8_t* remb_img = nullptr;    // activation images and targets of the embedding forward (fast path)
   int64_t ring_enqueued = 0;     // records appended (host order); the device count is st->ring_count
   // feature bounds of the ring (Algorithm 4 [l, u]): staged by ls_refresh_bounds,
   // published by ls_publish into pub[b].bounds
@@ -516,6 +517,8 @@ void train_fast_bind(const MlpDesc& m, TrainFast& f, uint8_t* base, float* parts
 cudaError_t train_fast_images(Ctx& c, cudaStream_t s);
 cudaError_t run_train_fast(Ctx& c, int batch, const int32_t* idx, int opt, float lr, float* loss_out,
                            cudaStream_t s);
+int64_t replay_embed_bytes(const MlpDesc& m, const TrainFast& f, int64_t rows);
+cudaError_t replay_embed_fast(Ctx& c, int64_t P, int64_t Rc, cudaStream_t s);
 bool plan_train_f32(const MlpDesc& m, int64_t n_params, int max_batch, int sms, int64_t* part_floats);
 cudaError_t run_train_f32(Ctx& c, int batch, const int32_t* idx, int opt, float lr, float* loss_out,
                           cudaStream_t s);

@@ -6,10 +6,13 @@
 // FIFO evicted, stream position p at row C + p mod P), [C + P, C + P + Rc)
 // replay pool.  One admission round (run_replay_admit):
 //   1. embedding rows: candidates t < P (pending positions not yet
-//      considered, in stream order) then kept records k < Rc; chunks of the
-//      training batch size go through k_replay_gather (z-score, bf16 rounding
-//      in bf16 mode), the training forward, and k_replay_embed
-//      (g = (yhat - y) a_last, |bf16(g)|^2, +inf for rows not in use);
+//      considered, in stream order) then kept records k < Rc, on the training
+//      step's operand images (replay_embed_fast: gather, hidden layers, the
+//      embedding rows), or, where that path does not
+//      apply, chunks of the training batch size through k_replay_gather
+//      (z-score, bf16 rounding in bf16 mode), the training forward, and
+//      k_replay_embed; g = (yhat - y) a_last, |bf16(g)|^2, +inf for rows not
+//      in use;
 //   2. nearest-neighbour distances on tensor cores (launch_rowmin_tc: bf16
 //      products, fp32 sums, row minima per CTA) or on CUDA cores for small
 //      shapes (k_rowmin_simt), minima combined by k_rowmin_reduce;
@@ -58,7 +61,7 @@ __global__ void k_replay_prep(ReplayGeom g, const DevState* st, int B, int nchun
   int64_t lo, hi;
   pending_range(st, g, lo, hi);
   const int64_t m = hi - lo, nr = *reinterpret_cast<const volatile int64_t*>(&st->replay_count);
-  if (threadIdx.x == 0) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
     counts[0] = m;
     counts[1] = nr;
     for (int c = 0; c < nchunks; ++c) {
@@ -66,7 +69,8 @@ __global__ void k_replay_prep(ReplayGeom g, const DevState* st, int B, int nchun
       counts[2 + c] = v < 0 ? 0 : (v > B ? B : v);
     }
   }
-  for (int64_t r = threadIdx.x; r < g.P + g.Rc; r += blockDim.x) {
+  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < g.P + g.Rc;
+       r += (int64_t)gridDim.x * blockDim.x) {
     norm[r] = INFINITY;
     rank[r] = 0;
   }
@@ -469,11 +473,15 @@ cudaError_t run_replay_admit(Ctx& c, float* d_out, float* n_out, cudaStream_t s)
   // 1. embeddings of the round's records (compact rows), in chunks of the training batch size
   const int nchunks = (int)((rows + Bc - 1) / Bc);
   e = traced(c, TR_REPLAY, 1, s, [&] {
-    k_replay_prep<<<1, 1024, 0, s>>>(g, c.st, Bc, nchunks, c.rcount, c.rnorm, c.rrank);
+    k_replay_prep<<<grid_for(rows, c.sms), 256, 0, s>>>(g, c.st, Bc, nchunks, c.rcount, c.rnorm, c.rrank);
     return cudaGetLastError();
   });
   if (e != cudaSuccess) return e;
-  for (int64_t row0 = 0; row0 < rows; row0 += Bc) {
+  if (c.remb_img) {
+    e = replay_embed_fast(c, g.P, g.Rc, s);
+    if (e != cudaSuccess) return e;
+  }
+  for (int64_t row0 = 0; !c.remb_img && row0 < rows; row0 += Bc) {
     const int B = (int)std::min<int64_t>(Bc, rows - row0);
     const int64_t* chunk_rows = c.rcount + 2 + row0 / Bc;
     e = traced(c, TR_REPLAY, 1, s, [&] {

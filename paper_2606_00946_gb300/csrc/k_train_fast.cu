@@ -101,6 +101,10 @@ struct TrArgs {
   const DevState* st;                // optimiser step counter (dropout stream)
   uint64_t drop_seed, drop_thr;      // keep <=> (u >> 11) >= drop_thr
   float drop_scale;                  // fp32 1 / (1 - p)
+  // replay admission's forward (EMB): records in use of the candidates' tiles
+  // and of the kept records' after them; tiles past them are skipped
+  const int64_t* counts;
+  int tiles_cand;
 };
 
 __device__ __forceinline__ uint16_t bf16_bits(float x) {
@@ -155,7 +159,9 @@ __device__ __forceinline__ void store_col16p(uint8_t* imgT, int rowsT, int r, in
 // rows (r the thread's row): Z + b, ReLU and, with `drop`, dropout of unit
 // n0 + c under the stream h1 (key rowkey + c, rowkey = (row << 20) | n0),
 // each activation rounded to bf16 once as packed pairs that both images take
-// their bytes from, and the 16-bit masks [Z > 0 and kept].
+// their bytes from, and the 16-bit masks [Z > 0 and kept].  EMB (a forward with
+// no backward): the row-major image alone.
+template <bool EMB>
 __device__ __forceinline__ void fwd_cols(uint32_t taddr, const float* s_bias, int cbeg, int cw, uint8_t* S1,
                                          uint8_t* S2, int NT, int r, uint16_t* mask_out, int64_t rows_pad,
                                          bool drop, uint64_t h1, uint64_t rowkey, uint64_t drop_thr,
@@ -189,9 +195,11 @@ __device__ __forceinline__ void fwd_cols(uint32_t taddr, const float* s_bias, in
       w[2 * g] = pack2(a4[0], a4[1]);
       w[2 * g + 1] = pack2(a4[2], a4[3]);
     }
-    mask_out[(int64_t)(c >> 4) * rows_pad] = (uint16_t)bits;
     store_row16p(S1, kM, r, c, w);
-    store_col16p(S2, NT, r, c, w);
+    if (!EMB) {
+      mask_out[(int64_t)(c >> 4) * rows_pad] = (uint16_t)bits;
+      store_col16p(S2, NT, r, c, w);
+    }
   }
 }
 
@@ -273,7 +281,7 @@ __device__ __forceinline__ void tr_tile_copies(const TrArgs& args, int bid, uint
 // the tile's image stores to reach global memory (other CTAs of the grid read
 // them); otherwise only until they have read shared memory.  Returns false
 // after a timed-out wait (error latched, copies in flight waited for).
-template <bool RING>
+template <bool RING, bool EMB = false>
 __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* smem, uint32_t tmem, uint32_t par,
                                         bool drain, bool copied) {
   const bool second = bid >= args.n_cta0;
@@ -375,7 +383,7 @@ __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* sm
     }
     uint16_t* mask_out = J.mask_out + j + (int64_t)(n0 >> 4) * J.rows_pad;
     const bool drop = J.drop_h > 0;
-    fwd_cols(tmem + lane_addr, s_bias, cbeg, cw, S1, S2, NT, r, mask_out, J.rows_pad, drop, h1,
+    fwd_cols<EMB>(tmem + lane_addr, s_bias, cbeg, cw, S1, S2, NT, r, mask_out, J.rows_pad, drop, h1,
              ((uint64_t)j << 20) | (uint64_t)n0, args.drop_thr, args.drop_scale);
   } else if (ok && J.epi == TE_DX) {
     for (int c = cbeg; c < cbeg + cw; c += 16) {
@@ -399,7 +407,7 @@ __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* sm
     for (int c = tid; c < NT; c += kT)
       J.colpart[(int64_t)mt * N + n0 + c] = ((red[c] + red[256 + c]) + red[512 + c]) + red[768 + c];
   }
-  if (J.epi == TE_FWD_OUT) {
+  if (!EMB && J.epi == TE_FWD_OUT) {
     // pass 1: activations and this warp's part of the output dot product
     // With all 256 columns in one CTA (no cluster), each warp keeps its two
     // 32-column halves apart and the row dot is added as the two 128-column
@@ -505,14 +513,14 @@ __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* sm
       }
     }
   }
-  if (ok && (J.epi == TE_FWD || J.epi == TE_DX || J.epi == TE_FWD_OUT)) {
+  if (ok && J.epi != TE_STORE) {
     fence_async_smem();  // staged tiles are read by the bulk copies (async proxy)
     __syncthreads();
     if (tid == 0) {
       if (J.out)
         for (int kb = 0; kb < NT / 64; ++kb)
           bulk_s2g(J.out + ((int64_t)(n0 / 64 + kb) * J.rows_pad + m0) * 128, S1 + (size_t)kb * kM * 128, kM * 128);
-      for (int h = 0; h < kM / 64; ++h)
+      for (int h = 0; !EMB && h < kM / 64; ++h)
         bulk_s2g(J.outT + ((int64_t)(m0 / 64 + h) * J.rT + n0) * 128, S2 + (size_t)h * NT * 128,
                  (uint32_t)NT * 128);
       if (drain) bulk_commit_wait_all();
@@ -525,9 +533,16 @@ __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* sm
 }
 
 // One launch per product (or pair of products): CTA b runs tile b.
-template <bool RING>
+template <bool RING, bool EMB>
 __global__ void __launch_bounds__(kT, 1) k_tr_gemm(const __grid_constant__ TrArgs args) {
   extern __shared__ uint8_t smem_raw[];
+  if (EMB) {  // the tile's rows are in use?  (the counts come from an earlier kernel)
+    pdl_trigger();
+    pdl_wait();
+    const int mt = (int)blockIdx.x / args.job[0].n_split;
+    const bool kept = mt >= args.tiles_cand;
+    if ((int64_t)(kept ? mt - args.tiles_cand : mt) * kM >= args.counts[kept ? 1 : 0]) return;
+  }
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* full = reinterpret_cast<uint64_t*>(tr_tail(smem));
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(full + 2 * kMaxChunks + 1);
@@ -554,11 +569,11 @@ __global__ void __launch_bounds__(kT, 1) k_tr_gemm(const __grid_constant__ TrArg
   // (it lets its successor in at its end), so after the previous step's
   // optimiser has completed: the weight images and the master read before
   // the wait below are final.
-  pdl_trigger();
+  if (!EMB) pdl_trigger();
   tr_tile_pre<RING>(args, (int)blockIdx.x, smem, false);
   // the activation and gradient operands come from the previous kernels of the
   // stream: their copies start as soon as the wait returns
-  pdl_wait();
+  if (!EMB) pdl_wait();
   if (threadIdx.x == 0) tr_tile_copies<RING>(args, (int)blockIdx.x, smem);
   tc_fence_before();
   __syncthreads();
@@ -566,7 +581,7 @@ __global__ void __launch_bounds__(kT, 1) k_tr_gemm(const __grid_constant__ TrArg
   const uint32_t tmem = *tmem_holder;
   // image stores may still be in flight when the CTA exits: the grid's
   // completion makes them visible to the next kernel
-  tr_tile<RING>(args, (int)blockIdx.x, smem, tmem, 0, false, true);
+  tr_tile<RING, EMB>(args, (int)blockIdx.x, smem, tmem, 0, false, true);
   if (threadIdx.x < 32) tmem_dealloc(tmem, tcols);
 }
 
@@ -968,17 +983,22 @@ TrArgs tr_args(const Ctx& c, const TrJob& j0, const TrJob* j1, int* err) {
   return a;
 }
 
-cudaError_t launch_tr_gemm(const Ctx& c, const TrJob& j0, const TrJob* j1, int* err, cudaStream_t s) {
-  const TrArgs a = tr_args(c, j0, j1, err);
+cudaError_t launch_tr_args(const Ctx& c, const TrArgs& a, bool emb, cudaStream_t s) {
+  const TrJob& j0 = a.job[0];
   const int n = a.n_cta;
   const int smem = gemm_smem_bytes();
-  auto* k = c.tf.wide ? k_tr_gemm<true> : k_tr_gemm<false>;
+  auto* k = emb ? (c.tf.wide ? k_tr_gemm<true, true> : k_tr_gemm<false, true>)
+                : (c.tf.wide ? k_tr_gemm<true, false> : k_tr_gemm<false, false>);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   // the column parts of a TE_FWD_OUT tile exchange row sums through
   // distributed shared memory: one cluster per tile
-  const int cl = (j0.epi == TE_FWD_OUT && !j1) ? j0.n_split : 1;
+  const int cl = j0.epi == TE_FWD_OUT ? j0.n_split : 1;
   return launch_chained(k, dim3(n), dim3(kT), (size_t)smem, s, cl, a);
+}
+
+cudaError_t launch_tr_gemm(const Ctx& c, const TrJob& j0, const TrJob* j1, int* err, cudaStream_t s) {
+  return launch_tr_args(c, tr_args(c, j0, j1, err), false, s);
 }
 
 // Column parts per tile of a product with N columns: two when the columns
@@ -1313,6 +1333,216 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
   return traced(c, TR_OPT, 1, s, [&] {
     const int grid = opt_blocks(m, a);
     return launch_chained(k_tr_opt, dim3(grid), dim3(256), 0, s, 1, a);
+  });
+}
+
+// ---------------------------------------------------------------------------
+// Replay admission's embeddings on the operand images (k_replay.cu)
+// ---------------------------------------------------------------------------
+namespace {
+
+struct EmbGather {
+  int rows, tiles_cand, d, d_pad;  // rows of the image: the candidates' tiles, then the kept records'
+  int64_t C, P, base;              // FIFO and pending capacities, first replay row
+  const int64_t* counts;           // candidates, kept records
+  const DevState* st;
+  const float* ring_x;
+  const float* ring_y;
+  const float* mean;
+  const float* stdv;
+  uint8_t* a0;
+  float* y;
+};
+
+// Image rows of the round's records, z-scored and rounded to bf16 (thread =
+// (row, 8 columns)); rows past a tile's records are zero, tiles past them are
+// left alone.
+__global__ void __launch_bounds__(256) k_emb_gather(const __grid_constant__ EmbGather g) {
+  pdl_wait();
+  pdl_trigger();
+  const int64_t m = g.counts[0], nr = g.counts[1];
+  const int64_t count = g.st->ring_count, hi = count > g.C ? count - g.C : 0, lo = hi - m;
+  const int rc = g.tiles_cand * kM;
+  const bool vec = (g.d & 3) == 0;
+  const int total = g.rows * (g.d_pad / 8);
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+    const int j = e % g.rows, c0 = (e / g.rows) * 8;
+    const int64_t i = j < rc ? j : j - rc, used = j < rc ? m : nr;
+    if ((i & ~(int64_t)(kM - 1)) >= used) continue;
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = 0.0f;
+    float y = 0.0f;
+    if (i < used) {
+      const int64_t slot = j < rc ? g.C + (lo + i) % g.P : g.base + i;
+      const float* row = g.ring_x + slot * g.d;
+      if (vec && c0 + 8 <= g.d) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float4 xv = __ldg(reinterpret_cast<const float4*>(row + c0) + h);
+          const float4 mv = __ldg(reinterpret_cast<const float4*>(g.mean + c0) + h);
+          const float4 sv = __ldg(reinterpret_cast<const float4*>(g.stdv + c0) + h);
+          v[4 * h] = zscore(xv.x, mv.x, sv.x);
+          v[4 * h + 1] = zscore(xv.y, mv.y, sv.y);
+          v[4 * h + 2] = zscore(xv.z, mv.z, sv.z);
+          v[4 * h + 3] = zscore(xv.w, mv.w, sv.w);
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (c0 + u < g.d) v[u] = zscore(__ldg(row + c0 + u), __ldg(g.mean + c0 + u), __ldg(g.stdv + c0 + u));
+      }
+      if (c0 == 0) y = g.ring_y[slot];
+    }
+    if (c0 == 0) g.y[j] = y;
+    *reinterpret_cast<uint4*>(g.a0 + sw128_offset(j, c0, g.rows)) =
+        make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
+  }
+}
+
+// The gradient embeddings of the round, a warp per image row: yhat from the
+// last hidden activations (bf16 weights, lanes along them), g = (yhat - y) a
+// in bf16 into the embedding image (tiles of 128 rows, a tile's K-blocks
+// together) and |bf16(g)|^2 of the rows in use, every sum in the order of the
+// general path's k_out_fwd and k_replay_embed.
+struct EmbRows {
+  int rows, tiles_cand, H;
+  int64_t P;
+  const int64_t* counts;
+  const uint8_t* a;  // image of the last hidden activations
+  const float* w;    // output layer
+  const float* b;
+  const float* y;
+  uint8_t* img;
+  float* norm;       // [P] candidates, then kept records
+};
+
+__global__ void __launch_bounds__(256) k_emb_rows(const __grid_constant__ EmbRows g) {
+  pdl_wait();
+  pdl_trigger();
+  const int lane = threadIdx.x & 31, rc = g.tiles_cand * kM;
+  const int64_t m = g.counts[0], nr = g.counts[1];
+  for (int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < g.rows; j += (gridDim.x * blockDim.x) >> 5) {
+    const bool kept = j >= rc;
+    const int64_t i = kept ? j - rc : j, used = kept ? nr : m;
+    if ((i & ~(int64_t)(kM - 1)) >= used) continue;  // a tile without records
+    float av[8], z = 0.0f;  // H <= 256
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int k = lane + 32 * u;
+      av[u] = k < g.H ? __uint_as_float((uint32_t)*reinterpret_cast<const uint16_t*>(g.a + sw128_offset(j, k, g.rows)) << 16)
+                      : 0.0f;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (lane + 32 * u < g.H) z = fmaf(av[u], round_bf16(__ldg(g.w + lane + 32 * u)), z);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+    const float res = (z + __ldg(g.b)) - g.y[j];
+    uint8_t* tile = g.img + (int64_t)(j / kM) * kM * g.H * 2;
+    float s = 0.0f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int k = lane + 32 * u;
+      if (k >= g.H) break;
+      const uint16_t b = bf16_bits(res * av[u]);
+      const float bv = __uint_as_float((uint32_t)b << 16);
+      s = fmaf(bv, bv, s);
+      *reinterpret_cast<uint16_t*>(tile + sw128_offset(j % kM, k, kM)) = b;
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0 && i < used) g.norm[(kept ? g.P : 0) + i] = s;
+  }
+}
+
+// Widest image of the embedding forward: layer inputs and the last hidden
+// activations.
+int emb_width(const MlpDesc& m, const TrainFast& f) {
+  int w = m.w[m.n_layers - 1];
+  for (int l = 0; l + 1 < m.n_layers; ++l) w = std::max(w, f.in_pad[l]);
+  return w;
+}
+
+}  // namespace
+
+// Bytes of the two activation images and the targets of an admission round
+// over `rows` image rows (0: the embeddings run through the general forward).
+int64_t replay_embed_bytes(const MlpDesc& m, const TrainFast& f, int64_t rows) {
+  return f.on ? 2 * rows * emb_width(m, f) * 2 + rows * 4 : 0;
+}
+
+// Embeddings of the round whose counts and reset norms k_replay_prep left:
+// gather, the hidden layers, the embedding rows.  (In chunks of the training
+// batch through the general forward, fp32 operands staged by every product:
+// 15 launches for pools of 5000; an admission round of 1000 candidates took
+// 160 us, 65 us on the images.)
+cudaError_t replay_embed_fast(Ctx& c, int64_t P, int64_t Rc, cudaStream_t s) {
+  const MlpDesc& m = c.mlp;
+  TrainFast& f = c.tf;
+  const int nh = m.n_layers - 1;
+  const int tc = (int)((P + kM - 1) / kM), T = tc + (int)((Rc + kM - 1) / kM), rows = T * kM;
+  const int pad = emb_width(m, f);
+  uint8_t* img[2] = {c.remb_img, c.remb_img + (int64_t)rows * pad * 2};
+  float* y = reinterpret_cast<float*>(c.remb_img + 2 * (int64_t)rows * pad * 2);
+  EmbGather g{};
+  g.rows = rows;
+  g.tiles_cand = tc;
+  g.d = m.w[0];
+  g.d_pad = f.in_pad[0];
+  g.C = c.cfg.ring_capacity;
+  g.P = P;
+  g.base = c.replay_base;
+  g.counts = c.rcount;
+  g.st = c.st;
+  g.ring_x = c.ring_x;
+  g.ring_y = c.ring_y;
+  g.mean = c.mean;
+  g.stdv = c.stdv;
+  g.a0 = img[0];
+  g.y = y;
+  cudaError_t e = traced(c, TR_REPLAY, 1, s, [&] {
+    const int64_t total = (int64_t)rows * (g.d_pad / 8);
+    const int grid = (int)std::min<int64_t>((total + 255) / 256, (int64_t)c.sms * 8);
+    return launch_chained(k_emb_gather, dim3(grid), dim3(256), 0, s, 1, g);
+  });
+  for (int l = 0; e == cudaSuccess && l < nh; ++l) {
+    const int N = m.w[l + 1];
+    TrJob J{};
+    J.epi = TE_FWD;
+    J.m_tiles = T;
+    J.n_split = n_split_fwd(N, T, c.sms);
+    J.splits = 1;
+    J.nchunks = J.kblocks = f.in_pad[l] / 64;
+    J.NT = N / J.n_split;
+    J.A = img[l & 1];
+    J.rA = rows;
+    J.B = f.imgW[l];
+    J.M = rows;
+    J.bias = c.master + m.boff[l];
+    J.rows_pad = rows;
+    J.out = img[(l + 1) & 1];
+    TrArgs a = tr_args(c, J, nullptr, c.d_err);
+    a.counts = c.rcount;
+    a.tiles_cand = tc;
+    e = traced(c, TR_REPLAY, 1, s, [&] { return launch_tr_args(c, a, true, s); });
+  }
+  if (e != cudaSuccess) return e;
+  EmbRows r{};
+  r.rows = rows;
+  r.tiles_cand = tc;
+  r.H = m.w[nh];
+  r.P = P;
+  r.counts = c.rcount;
+  r.a = img[nh & 1];
+  r.w = c.master + m.woff[nh];
+  r.b = c.master + m.boff[nh];
+  r.y = y;
+  r.img = c.rimg;
+  r.norm = c.rnorm;
+  return traced(c, TR_REPLAY, 1, s, [&] {
+    const int grid = std::min((rows + 7) / 8, c.sms * 8);
+    return launch_chained(k_emb_rows, dim3(grid), dim3(256), 0, s, 1, r);
   });
 }
 
