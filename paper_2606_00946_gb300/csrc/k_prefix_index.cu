@@ -13,7 +13,10 @@
 // recurrence), looks the 32 keys up at once, and a warp-wide prefix AND of
 // their instance masks gives, per lane, the instances still matching every
 // block up to it.  An instance that stops matching in the round gets its hit
-// length from one ballot; the lane that owns the instance keeps it and the
+// length from one ballot, or, when several of a group of 32 stop in it, from a
+// bit transpose of their alive masks (a request's first blocks end most of the
+// instances: at 256 instances the ballots, a dozen instructions each, were
+// most of a walk's first round).  The hit lengths wait in shared memory and the
 // row is written once, coalesced, at the end.  The walk stops at the first
 // round after which no instance matches, so tokens past the longest hit plus
 // one round are never read.  Walks differ in length by orders of magnitude,
@@ -27,6 +30,7 @@ namespace {
 using namespace bh;
 
 constexpr int kNT = 128;
+constexpr int kFewDeaths = 2;  // instances of 32 that end in a round one by one; more, by a transpose
 
 // Slot of `key` in the index (linear probing in aligned 4-slot buckets), -1 if absent.
 __device__ __forceinline__ int64_t index_find(const uint64_t* __restrict__ gkeys, uint64_t gmask_slots,
@@ -72,6 +76,19 @@ __device__ __forceinline__ uint64_t index_mask_w1(const uint64_t* __restrict__ e
   return 0;
 }
 
+// Transpose of the warp's 32 x 32 bit matrix: bit b of lane i of the result is
+// bit i of lane b's v.
+__device__ __forceinline__ uint32_t transpose32(uint32_t v, int lane) {
+#pragma unroll
+  for (int j = 16; j; j >>= 1) {
+    const uint32_t m = j == 16 ? 0x0000ffffu : j == 8 ? 0x00ff00ffu : j == 4 ? 0x0f0f0f0fu : j == 2 ? 0x33333333u
+                                                                                           : 0x55555555u;
+    const uint32_t y = __shfl_xor_sync(kFull, v, j);
+    v = (lane & j) ? (v & ~m) | ((y >> j) & m) : (v & m) | ((y & m) << j);
+  }
+  return v;
+}
+
 template <int W>
 __global__ void __launch_bounds__(kNT, W <= 4 ? 8 : 1) k_prefix_index(int n_req, const int32_t* __restrict__ tok,
                                                       const int64_t* __restrict__ tok_off,
@@ -85,6 +102,10 @@ __global__ void __launch_bounds__(kNT, W <= 4 ? 8 : 1) k_prefix_index(int n_req,
   // G^(lane+1): the factor by which the state entering a round reaches lane
   // `lane` (kept in shared memory: one load per round, no registers held)
   __shared__ uint64_t s_glane[32];
+  // hit lengths of the instances that ended in this warp's walk (each written
+  // and read by the lane i mod 32)
+  __shared__ int32_t s_ended[kNT / 32][64 * W];
+  int32_t* const ended = s_ended[threadIdx.x >> 5];
   if (threadIdx.x < 32) {
     uint64_t g = 1, b = kG;
     for (unsigned e = (unsigned)lane + 1; e; e >>= 1) {
@@ -101,12 +122,10 @@ __global__ void __launch_bounds__(kNT, W <= 4 ? 8 : 1) k_prefix_index(int n_req,
     const uintptr_t ab = reinterpret_cast<uintptr_t>(base);
     const int align = (ab & 15) == 0 ? 16 : (ab & 7) == 0 ? 8 : 4;
     uint64_t alive[W];
-    int32_t hreg[W][2];  // hit length of instances 64w + lane and 64w + 32 + lane
 #pragma unroll
     for (int w = 0; w < W; ++w) {
       const int lo = 64 * w;
       alive[w] = n_inst >= lo + 64 ? ~0ull : (n_inst > lo ? ((1ull << (n_inst - lo)) - 1ull) : 0ull);
-      hreg[w][0] = hreg[w][1] = 0;
     }
     uint64_t state = kG;  // s_{-1}
     bool any = n_inst > 0;
@@ -151,15 +170,20 @@ __global__ void __launch_bounds__(kNT, W <= 4 ? 8 : 1) k_prefix_index(int n_req,
         }
         x &= alive[w];
         const uint64_t end = __shfl_sync(kFull, x, 31);
-        uint64_t died = alive[w] & ~end;
-        while (died) {
-          const int bit = __ffsll((long long)died) - 1;
-          const int cnt = __popc(__ballot_sync(kFull, (x >> bit) & 1ull));
-          if (lane == (bit & 31)) {
-            if (bit >> 5) hreg[w][1] = (int32_t)(p + cnt);
-            else hreg[w][0] = (int32_t)(p + cnt);
+        const uint64_t died = alive[w] & ~end;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          uint32_t d = (uint32_t)(died >> (32 * h));
+          if (__popc(d) > kFewDeaths) {
+            const int cnt = __popc(transpose32((uint32_t)(x >> (32 * h)), lane));
+            if ((d >> lane) & 1u) ended[64 * w + 32 * h + lane] = (int32_t)(p + cnt);
+          } else {
+            for (; d; d &= d - 1) {
+              const int bit = __ffs(d) - 1;
+              const int cnt = __popc(__ballot_sync(kFull, (x >> (32 * h + bit)) & 1ull));
+              if (lane == bit) ended[64 * w + 32 * h + lane] = (int32_t)(p + cnt);
+            }
           }
-          died &= died - 1;
         }
         alive[w] = end;
         any = any || end != 0;
@@ -172,7 +196,7 @@ __global__ void __launch_bounds__(kNT, W <= 4 ? 8 : 1) k_prefix_index(int n_req,
       for (int h = 0; h < 2; ++h) {
         const int bit = 32 * h + lane, i = 64 * w + bit;
         // instances matching every full block (or requests without a full block)
-        if (i < n_inst) hrow[i] = ((alive[w] >> bit) & 1ull) ? (int32_t)nb : hreg[w][h];
+        if (i < n_inst) hrow[i] = ((alive[w] >> bit) & 1ull) ? (int32_t)nb : ended[i];
       }
     // the next request: from the counter (after each warp's first), else a fixed stride
     if (st) {
