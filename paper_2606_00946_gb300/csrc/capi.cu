@@ -117,7 +117,7 @@ void free_all(Ctx& c) {
                   c.gpart, c.loss_tmp, c.d_err, c.pub[0].img, c.pub[1].img, c.xin, c.xrq, c.pairx, c.ximg,
                   c.bkeys, c.work, c.work_n, c.gkeys, c.gmask, c.st, c.tf.base, c.tf.parts,
                   c.pub[0].bounds, c.pub[1].bounds, c.bounds_stage, c.benc, c.remb, c.rnorm, c.rpart, c.rd,
-                  c.rn, c.rinv, c.rcount, c.rimg, c.rrank, c.tr_bar, c.trs_part, c.remb_img};
+                  c.rn, c.rinv, c.rcount, c.rimg, c.rrank, c.tr_bar, c.trs_part, c.remb_img, c.order};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c.ev_pub) cudaEventDestroy(c.ev_pub);
@@ -242,6 +242,7 @@ int ls_create(const ls_config* cfg, ls_ctx** out) {
     A(dalloc(&c.work, R * NI));
   } else if (c.use_index) {
     A(dalloc(&c.bkeys, c.bkeys_cap));  // block keys of a sequential-commit batch
+    A(dalloc(&c.order, R));
   }
   A(dalloc(&c.work_n, 1));
   A(dalloc(&c.xin, NI * std::max(1, c.tc.d_pad)));
@@ -582,7 +583,7 @@ int route_impl(ls_ctx* h, int32_t n_req, const int32_t* tok, const int64_t* tok_
   if (c.use_index) {
     LS_CK(traced(c, TR_PREFIX_INDEX, 1, s, [&] {
       return launch_prefix_index(n_req, tok, tok_off, c.gkeys, c.gmask, c.gW, (uint64_t)(c.gslots - 1), c.n_inst,
-                                 hits, c.sms, c.st, s);
+                                 hits, c.order, c.sms, c.st, s);
     }));
   } else if (c.cfg.prefix_mode == LS_PREFIX_FUSED) {
     LS_CK(traced(c, TR_PREFIX, 1, s, [&] {

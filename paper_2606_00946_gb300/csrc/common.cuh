@@ -253,6 +253,7 @@ struct Ctx {
   int64_t gslots = 0;
   uint64_t* gkeys = nullptr;  // [gslots]
   uint64_t* gmask = nullptr;  // [gslots, gW]
+  uint32_t* order = nullptr;  // requests of the batch by falling length [max_requests] (index walk)
   uint64_t* bkeys = nullptr;  // block keys of the batch, slot tok_off[r]/16 + b
   int64_t bkeys_cap = 0;
   uint32_t* work = nullptr;   // (request, instance) pairs that hit block 0
@@ -525,7 +526,7 @@ cudaError_t run_train_f32(Ctx& c, int batch, const int32_t* idx, int opt, float 
 void set_last_error(const char* msg);  // sets the text ls_last_error() returns
 cudaError_t launch_prefix_index(int n_req, const int32_t* tok, const int64_t* tok_off, const uint64_t* gkeys,
                                 const uint64_t* gmask, int W, uint64_t gmask_slots, int n_inst, int32_t* hits,
-                                int sms, DevState* st, cudaStream_t s);
+                                uint32_t* order, int sms, DevState* st, cudaStream_t s);
 cudaError_t launch_index_insert(const uint64_t* keys, const int64_t* key_off, int n_inst, int64_t n_keys,
                                 uint64_t* gkeys, uint64_t* gmask, int W, uint64_t gmask_slots, int32_t* counts,
                                 int64_t max_keys, int* err, int sms, cudaStream_t s);
