@@ -577,7 +577,7 @@ int route_impl(ls_ctx* h, int32_t n_req, const int32_t* tok, const int64_t* tok_
   if (weight_version_out) *weight_version_out = v;
   if (n_req == 0) return LS_OK;
   int32_t* hits = hits_opt ? hits_opt : c.hits;
-  const bool fused_select = !guarded && (c.use_tc ? scorer_selects(c.tc, c.n_inst)
+  const bool fused_select = !guarded && (c.use_tc ? scorer_selects(c.tc, n_req, c.n_inst)
                                                   : simt_selects(c.mlp, n_req, c.n_inst, c.sms));
   float* scores = scores_opt ? scores_opt : (fused_select ? nullptr : c.scores);
   if (c.use_index) {

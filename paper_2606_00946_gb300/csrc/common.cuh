@@ -479,9 +479,15 @@ cudaError_t launch_inst_templates(int n_inst, int d_inst, const float* inst, con
 cudaError_t launch_feature_image(const int64_t* tok_off, const int32_t* hits, int n_inst, const uint16_t* xin,
                                  int d_inst, int n_req, int d_req, const float* req, const float* mean,
                                  const float* stdv, int d_pad, uint8_t* ximg, int sms, cudaStream_t s);
-// With the pipelined kernel and n_inst dividing 32 the selector runs inside the
-// scorer (choice/best written, scores only when non-NULL); see scorer_selects().
-inline bool scorer_selects(const TcPlan& p, int n_inst) { return p.pipe && n_inst <= 32 && 32 % n_inst == 0; }
+// The selector runs inside the scorer (choice/best written, scores only when
+// non-NULL) with the pipelined kernel and n_inst dividing 32, and with the
+// generic kernel when its 128-row tiles hold whole requests: n_inst divides
+// 128, or the batch is one tile.
+inline bool scorer_selects(const TcPlan& p, int n_req, int n_inst) {
+  if (p.pipe) return n_inst <= 32 && 32 % n_inst == 0;
+  if (p.pair || p.wide) return false;
+  return (n_inst <= 128 && 128 % n_inst == 0) || (int64_t)n_req * n_inst <= 128;
+}
 cudaError_t launch_score_tc(const MlpDesc& m, const TcPlan& p, const Published* pub, const int32_t* sel,
                             int n_req, int n_inst, const uint4* pairx, const uint8_t* ximg, int32_t* choice,
                             float* best,

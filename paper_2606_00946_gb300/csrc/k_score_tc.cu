@@ -39,7 +39,7 @@ struct TcArgs {
   int n_req, n_inst, d, d_inst, d_req;
   const uint4* pairx;    // [rows] bf16 pair features (chunk 0 of each feature row, zeros past column 5)
   const uint8_t* ximg;   // pipelined kernel: feature tiles, tile t = xbytes at t * xbytes, in the MMA layout
-  int32_t* choice;       // pipelined kernel with n_inst dividing 32: the selector runs in the epilogue
+  int32_t* choice;       // with fuse_argmin (scorer_selects): the selector runs in the epilogue
   float* best;
   int fuse_argmin;
   const uint16_t* xin;   // [n_inst, d_pad] bf16 instance template rows (zero outside inst columns)
@@ -139,11 +139,19 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
 
 __device__ __forceinline__ float4 ldg4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
 
-__global__ void __launch_bounds__(kThreadsTc, 1) k_score_tc(const __grid_constant__ TcArgs a) {
+// Bound by its chain a tile: build, product, epilogue, next layer.  Two CTAs
+// share an SM when the weights and the operand tile take half its shared
+// memory, so that one's products and waits overlap the other's epilogues.
+// Whole routes of 64-128-128-128-1, with the selection and the chained launch
+// below: 4096 requests x 16 instances 40.8 -> 32.9 us, 5000 x 200 353 -> 242,
+// 16 x 64 21.9 -> 17.0.  A predictor too large for two (64-192-192-192-1) is
+// unchanged: 70.1 us for 4096 x 32 on either side.
+template <int PER_SM>
+__global__ void __launch_bounds__(kThreadsTc, PER_SM) k_score_tc(const __grid_constant__ TcArgs a) {
   const bool pb = a.sel && *a.sel == 1;  // published buffer of this route
   const uint8_t* __restrict__ img = pb ? a.img1 : a.img0;
   const float* __restrict__ params = pb ? a.params1 : a.params0;
-  extern __shared__ uint8_t smem_raw[];
+  extern __shared__ __align__(128) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const TcPlan& p = a.p;
   uint8_t* A = smem;
@@ -208,10 +216,13 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_score_tc(const __grid_constan
   const int cq = warp >> 2;  // column quarter handled by this warp
   const int row = 32 * q4 + lane;
   const uint32_t lane_addr = (uint32_t)(32 * q4) << 16;
+  // what precedes reads the published weights alone; the feature rows come
+  // from the previous kernel of the stream
+  pdl_wait();
 
   for (int it = 0; it < my_tiles; ++it) {
     const int64_t row0 = (int64_t)(blockIdx.x + (int64_t)it * gridDim.x) * kTileM;
-    build_tile<4>(a, A, row0, threadIdx.x, kThreadsTc);
+    build_tile<PER_SM == 1 ? 4 : 2>(a, A, row0, threadIdx.x, kThreadsTc);
     fence_async_smem();
     __syncthreads();
     if (*abort_flag) break;
@@ -308,13 +319,35 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_score_tc(const __grid_constan
         part[cq * kTileM + row] = sacc;
         tc_fence_before();
         __syncthreads();
+        float* sc = part + 4 * kTileM;  // the tile's predictions
         if (tid < kTileM) {
           const int64_t g = row0 + tid;
-          if (g < a.rows)
-            a.scores[g] = ((part[tid] + part[kTileM + tid]) + (part[2 * kTileM + tid] + part[3 * kTileM + tid])) +
+          const float y = ((part[tid] + part[kTileM + tid]) + (part[2 * kTileM + tid] + part[3 * kTileM + tid])) +
                           __ldg(params + a.p.b_last_off);
+          if (g < a.rows && a.scores) a.scores[g] = y;
+          sc[tid] = y;
         }
         __syncthreads();
+        if (a.fuse_argmin) {  // the tile holds whole requests: a warp selects for each
+          const int64_t r0 = row0 / a.n_inst;
+          const int nr = (int)((a.rows - row0 < kTileM ? a.rows - row0 : kTileM) / a.n_inst);
+          for (int r = warp; r < nr; r += kThreadsTc / 32) {
+            float bv = 0.0f;
+            int bi = -1;
+            for (int i = lane; i < a.n_inst; i += 32) {
+              const float v = sc[r * a.n_inst + i];
+              if (bi < 0 || score_precedes(v, i, bv, bi)) { bv = v; bi = i; }
+            }
+#pragma unroll
+            for (int o = 16; o; o >>= 1) {
+              const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+              const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+              if (oi >= 0 && (bi < 0 || score_precedes(ov, oi, bv, bi))) { bv = ov; bi = oi; }
+            }
+            if (lane == 0) { a.choice[r0 + r] = bi; a.best[r0 + r] = bv; }
+          }
+          __syncthreads();
+        }
       }
       if (*abort_flag) break;
     }
@@ -328,6 +361,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_score_tc(const __grid_constan
   }
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, p.tmem_cols);
+  pdl_trigger();
 }
 
 // ---------------------------------------------------------------------------
@@ -1479,51 +1513,81 @@ __global__ void __launch_bounds__(kThreadsPair, 1) k_score_pair(const __grid_con
 // and, for every (request, instance) pair, the 16-byte first chunk of its
 // feature row holding the six z-scored pair features (Sec. 4.1 Features;
 // Algorithm 4 Normalize) with zeros in columns 6 and 7.
+// The pair chunks bound it by their arithmetic (seven IEEE divisions a pair),
+// so what can be is kept out of the loop: the means and deviations, the
+// division that finds a thread's next pair's request, 64-bit conversions.
 template <typename I>  // index type: 32-bit when every index fits, else 64-bit
-__global__ void k_norm_rows(const int64_t* __restrict__ tok_off, const int32_t* __restrict__ hits,
-                            uint4* __restrict__ pairx, int n_inst, int d_inst, const float* __restrict__ inst,
-                            int n_req, int d_req, const float* __restrict__ req, const float* __restrict__ mean,
-                            const float* __restrict__ stdv, int d_pad, uint16_t* __restrict__ xin,
-                            uint16_t* __restrict__ xrq) {
-  // items: eight template columns of an instance row, of a request row, then
-  // one (request, instance) pair
+__global__ void __launch_bounds__(256) k_norm_rows(const int64_t* __restrict__ tok_off,
+                                                   const int32_t* __restrict__ hits, uint4* __restrict__ pairx,
+                                                   int n_inst, int d_inst, const float* __restrict__ inst, int n_req,
+                                                   int d_req, const float* __restrict__ req,
+                                                   const float* __restrict__ mean, const float* __restrict__ stdv,
+                                                   int d_pad, uint16_t* __restrict__ xin,
+                                                   uint16_t* __restrict__ xrq) {
+  pdl_wait();  // hit lengths from the prefix kernel
+  // eight template columns of an instance row or of a request row
   const I G = (I)(d_pad / 8);
-  const I ni = (I)n_inst * G, nr = (I)n_req * G, np = (I)n_req * (I)n_inst;
-  for (I e = (I)blockIdx.x * blockDim.x + threadIdx.x; e < ni + nr + np; e += (I)gridDim.x * blockDim.x) {
-    if (e < ni + nr) {
-      const bool is_inst = e < ni;
-      const I f = is_inst ? e : e - ni;
-      const I row = f / G;
-      const int c0 = (int)(f - row * G) * 8;
-      const int off = is_inst ? kPair : kPair + d_inst, dk = is_inst ? d_inst : d_req;
-      const float* src = is_inst ? inst + (int64_t)row * d_inst : req + (int64_t)row * d_req;
-      uint32_t w[4];
+  const I ni = (I)n_inst * G, nr = (I)n_req * G;
+  const I first = (I)blockIdx.x * blockDim.x + threadIdx.x, stride = (I)gridDim.x * blockDim.x;
+  for (I e = first; e < ni + nr; e += stride) {
+    const bool is_inst = e < ni;
+    const I f = is_inst ? e : e - ni;
+    const I row = f / G;
+    const int c0 = (int)(f - row * G) * 8;
+    const int off = is_inst ? kPair : kPair + d_inst, dk = is_inst ? d_inst : d_req;
+    const float* src = is_inst ? inst + (int64_t)row * d_inst : req + (int64_t)row * d_req;
+    uint32_t w[4];
 #pragma unroll
-      for (int u = 0; u < 8; u += 2) {
-        uint32_t pr = 0;
+    for (int u = 0; u < 8; u += 2) {
+      uint32_t pr = 0;
 #pragma unroll
-        for (int v = 0; v < 2; ++v) {
-          const int k = c0 + u + v - off;
-          const uint16_t b = (k >= 0 && k < dk) ? bf16_bits(zscore(src[k], mean[off + k], stdv[off + k])) : (uint16_t)0;
-          pr |= (uint32_t)b << (16 * v);
-        }
-        w[u / 2] = pr;
+      for (int v = 0; v < 2; ++v) {
+        const int k = c0 + u + v - off;
+        const uint16_t b = (k >= 0 && k < dk) ? bf16_bits(zscore(src[k], mean[off + k], stdv[off + k])) : (uint16_t)0;
+        pr |= (uint32_t)b << (16 * v);
       }
-      uint16_t* dst = (is_inst ? xin : xrq) + (int64_t)row * d_pad + c0;
-      *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-    } else {
-      const I g = e - ni - nr;
-      const I r = g / (I)n_inst;
-      const int64_t L = __ldg(tok_off + r + 1) - __ldg(tok_off + r);
-      const int h = __ldg(hits + g);
-      uint16_t f[kPair];
+      w[u / 2] = pr;
+    }
+    uint16_t* dst = (is_inst ? xin : xrq) + (int64_t)row * d_pad + c0;
+    *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+  float mu[kPair], sd[kPair];
 #pragma unroll
-      for (int k = 0; k < kPair; ++k)
-        f[k] = bf16_bits(zscore(raw_feature(k, L, h, nullptr, 0, nullptr), __ldg(mean + k), __ldg(stdv + k)));
-      pairx[g] = make_uint4(f[0] | ((uint32_t)f[1] << 16), f[2] | ((uint32_t)f[3] << 16),
-                            f[4] | ((uint32_t)f[5] << 16), 0u);
+  for (int k = 0; k < kPair; ++k) {
+    mu[k] = __ldg(mean + k);
+    sd[k] = __ldg(stdv + k);
+    sd[k] = sd[k] < 1e-12f ? 1.0f : sd[k];  // (as zscore takes it)
+  }
+  const I np = (I)n_req * (I)n_inst, N = (I)n_inst;
+  const I dr = stride / N, di = stride - dr * N;
+  I r = first / N, i = first - r * N;
+  for (I g = first; g < np; g += stride) {
+    const int64_t L = __ldg(tok_off + r + 1) - __ldg(tok_off + r);
+    const int h = __ldg(hits + g);
+    float x[kPair];
+    if (L >= 0 && L < (1 << 30) && h >= 0 && h < (1 << 26)) {  // every integer feature fits 32 bits
+      const int l = (int)L, t = kBlockTok * h;
+      x[0] = (float)l;
+      x[1] = (float)h;
+      x[2] = (float)t;
+      x[3] = l > 0 ? (float)t / (float)l : 0.0f;
+      x[4] = (float)(l - t);
+      x[5] = (float)((l + kBlockTok - 1) / kBlockTok - h);
+    } else {
+#pragma unroll
+      for (int k = 0; k < kPair; ++k) x[k] = raw_feature(k, L, h, nullptr, 0, nullptr);
+    }
+#pragma unroll
+    for (int k = 0; k < kPair; ++k) x[k] = (x[k] - mu[k]) / sd[k];
+    pairx[g] = make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]), 0u);
+    r += dr;
+    i += di;
+    if (i >= N) {
+      i -= N;
+      ++r;
     }
   }
+  pdl_trigger();  // the scorer may start once every CTA is here
 }
 
 // Instance template rows (computed when the snapshot or the normaliser
@@ -1663,7 +1727,7 @@ bool plan_tc(const MlpDesc& m, TcPlan& p, bool allow_pair, bool allow_pipe) {
     p.stages = std::min(smax, 8);
     if (p.stages < 2) return false;
   }
-  p.smem = p.a_bytes + p.stages * cb + (2 * p.stages + 1) * 8 + 16 + 1024;
+  p.smem = p.a_bytes + p.stages * cb + (2 * p.stages + 1) * 8 + 16 + 896;  // (a 128-byte aligned start)
   p.tmem_cols = 32;
   while ((int)p.tmem_cols < outmax) p.tmem_cols <<= 1;
   p.w_last_off = m.woff[m.n_layers - 1];
@@ -1813,13 +1877,9 @@ cudaError_t launch_norm_rows(const int64_t* tok_off, const int32_t* hits, uint4*
   const int64_t n = (int64_t)(n_inst + n_req) * d_pad + (int64_t)n_req * n_inst;
   if (n <= 0) return cudaSuccess;
   const int grid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)sms * 8);
-  if (n + (int64_t)grid * 256 < (1LL << 31))
-    k_norm_rows<uint32_t><<<grid, 256, 0, s>>>(tok_off, hits, pairx, n_inst, d_inst, inst, n_req, d_req, req, mean,
-                                               stdv, d_pad, xin, xrq);
-  else
-    k_norm_rows<int64_t><<<grid, 256, 0, s>>>(tok_off, hits, pairx, n_inst, d_inst, inst, n_req, d_req, req, mean,
-                                              stdv, d_pad, xin, xrq);
-  return cudaGetLastError();
+  auto* k = n + (int64_t)grid * 256 < (1LL << 31) ? k_norm_rows<uint32_t> : k_norm_rows<int64_t>;
+  return launch_chained(k, dim3(grid), dim3(256), 0, s, 1, tok_off, hits, pairx, n_inst, d_inst, inst, n_req, d_req,
+                        req, mean, stdv, d_pad, xin, xrq);
 }
 
 cudaError_t launch_inst_templates(int n_inst, int d_inst, const float* inst, const float* mean, const float* stdv,
@@ -1900,7 +1960,7 @@ cudaError_t launch_score_tc(const MlpDesc& m, const TcPlan& p, const Published* 
   a.ximg = ximg;
   a.choice = choice;
   a.best = best;
-  a.fuse_argmin = (p.pipe && choice && best && n_inst <= 32 && 32 % n_inst == 0) ? 1 : 0;
+  a.fuse_argmin = choice && best && scorer_selects(p, n_req, n_inst) ? 1 : 0;
   a.xin = xin;
   a.xrq = xrq;
   a.mean = mean;
@@ -1929,11 +1989,15 @@ cudaError_t launch_score_tc(const MlpDesc& m, const TcPlan& p, const Published* 
     if (e != cudaSuccess) return e;
     return launch_chained(k_score_wide, dim3(grid), dim3(kThreadsWide), (size_t)p.wide_smem, s, 1, a);
   } else {
-    cudaError_t e = cudaFuncSetAttribute(k_score_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+    if (!scores && !a.fuse_argmin) return cudaErrorInvalidValue;
+    // two CTAs an SM where shared memory and the 512 TMEM columns hold both
+    const bool two = p.smem <= 113 * 1024 && p.tmem_cols <= 256;
+    auto* kern = two ? k_score_tc<2> : k_score_tc<1>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
     if (e != cudaSuccess) return e;
-    k_score_tc<<<grid, kThreadsTc, p.smem, s>>>(a);
+    return launch_chained(kern, dim3(std::min(a.n_tiles, (two ? 2 : 1) * sms)), dim3(kThreadsTc), (size_t)p.smem, s, 1,
+                          a);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace ls
