@@ -168,12 +168,13 @@ struct Tracer {
 struct TrainFast {
   bool on = false;
   bool wide = false;                       // a hidden layer wider than 256 (chained launches only, no dropout)
+  int chain = 0;                           // forward and input gradients in one launch: CTAs per 128-row tile
   int rows_max = 0;                        // max_train_batch rounded up to 128
   int in_pad[LS_MAX_LAYERS] = {};          // K of layer l (input width padded to 64)
   uint8_t* imgA[LS_MAX_LAYERS] = {};       // A_l  [rows, in_pad[l]]
   uint8_t* imgAT[LS_MAX_LAYERS] = {};      // A_l^T [in_pad[l], rows]
   uint8_t* imgDZ[2] = {};                  // dz of a hidden layer [rows, width], by layer parity
-  uint8_t* imgDZT[2] = {};                 // its transpose [width padded to 128, rows]
+  uint8_t* imgDZT[LS_MAX_LAYERS] = {};     // its transpose [width padded to 128, rows], by layer (chain) or parity
   uint16_t* mask[LS_MAX_LAYERS + 1] = {};  // bits of [A_l > 0] as [width/16][rows]
   uint8_t* imgW[LS_MAX_LAYERS] = {};       // bf16 W_l  [out, in_pad]
   uint8_t* imgWT[LS_MAX_LAYERS] = {};      // bf16 W_l^T [in_pad, out]

@@ -141,6 +141,31 @@ __device__ __forceinline__ void store_row16p(uint8_t* img, int rows, int j, int 
   *reinterpret_cast<uint4*>(img + sw128_offset(j, c + 8, rows)) = make_uint4(w[4], w[5], w[6], w[7]);
 }
 
+// Where an epilogue's row-major columns go: a CTA's own tile (or nowhere).
+struct OwnRow {
+  uint8_t* S1;
+  __device__ __forceinline__ void operator()(int r, int c, const uint32_t (&w)[8]) const {
+    if (S1) store_row16p(S1, kM, r, c, w);
+  }
+};
+
+// The own tile and, in a cluster of two, the same place in the other CTA,
+// counted there on the K-block's barrier (the columns are those of whole
+// K-blocks).
+struct ClusterRow {
+  uint8_t* S1;
+  uint32_t peer, peer_bar;  // S1 and the barrier of its first K-block in the other CTA (0: none)
+  __device__ __forceinline__ void operator()(int r, int c, const uint32_t (&w)[8]) const {
+    if (!S1) return;
+    store_row16p(S1, kM, r, c, w);
+    if (peer) {
+      const uint32_t rb = peer_bar + 8 * (uint32_t)(c >> 6);
+      st_async_v4(peer + (uint32_t)sw128_offset(r, c, kM), w[0], w[1], w[2], w[3], rb);
+      st_async_v4(peer + (uint32_t)sw128_offset(r, c + 8, kM), w[4], w[5], w[6], w[7], rb);
+    }
+  }
+};
+
 // Transposed image [rowsT x 128] from packed bf16 pairs: element (c + u, r)
 // for u < 16, c % 16 == 0, r < 128 the tile row.  The same bytes as
 // sw128_offset(c + u, r, rowsT), with the row's swizzle phase (c + u) & 7 =
@@ -161,8 +186,8 @@ __device__ __forceinline__ void store_col16p(uint8_t* imgT, int rowsT, int r, in
 // each activation rounded to bf16 once as packed pairs that both images take
 // their bytes from, and the 16-bit masks [Z > 0 and kept].  EMB (a forward with
 // no backward): the row-major image alone.
-template <bool EMB>
-__device__ __forceinline__ void fwd_cols(uint32_t taddr, const float* s_bias, int cbeg, int cw, uint8_t* S1,
+template <bool EMB, class Row>
+__device__ __forceinline__ void fwd_cols(uint32_t taddr, const float* s_bias, int cbeg, int cw, const Row& row,
                                          uint8_t* S2, int NT, int r, uint16_t* mask_out, int64_t rows_pad,
                                          bool drop, uint64_t h1, uint64_t rowkey, uint64_t drop_thr,
                                          float drop_scale) {
@@ -195,10 +220,249 @@ __device__ __forceinline__ void fwd_cols(uint32_t taddr, const float* s_bias, in
       w[2 * g] = pack2(a4[0], a4[1]);
       w[2 * g + 1] = pack2(a4[2], a4[3]);
     }
-    store_row16p(S1, kM, r, c, w);
+    row(r, c, w);
     if (!EMB) {
       mask_out[(int64_t)(c >> 4) * rows_pad] = (uint16_t)bits;
       store_col16p(S2, NT, r, c, w);
+    }
+  }
+}
+
+// Epilogue scratch of a training-product CTA, after its barriers.
+struct EpiSmem {
+  static constexpr int kFloats = 256 + 256 + 8 * 256 + 8 * 128 + 128 + 128 + 8;
+  float* s_bias;  // [256]
+  float* s_w;     // [256] bf16-rounded output weights
+  float* red;     // [4][256] column sums by lane quadrant
+  float* red2;    // [4][256]
+  float* rowq;    // [8][128] row dots by column group
+  float* rowdot;  // [128] this CTA's row dots
+  float* yrow;    // [128] predictions
+  float* wsum;    // [8] warp partials
+  __device__ __forceinline__ explicit EpiSmem(uint8_t* at)
+      : s_bias(reinterpret_cast<float*>(at)),
+        s_w(s_bias + 256),
+        red(s_w + 256),
+        red2(red + 4 * 256),
+        rowq(red2 + 4 * 256),
+        rowdot(rowq + 8 * 128),
+        yrow(rowdot + 128),
+        wsum(yrow + 128) {}
+};
+
+// Column c's sum of the four lane quadrants' partials [4][256].
+__device__ __forceinline__ float col_total(const float* red, int c) {
+  return ((red[c] + red[256 + c]) + red[512 + c]) + red[768 + c];
+}
+
+// Input-gradient epilogue of one warp's columns: dz = acc [mask] sc, its
+// images (the row-major one through `row`) and the column sums of the 32 rows
+// into red.  mask_in: this row's 16-bit words, `stride` apart by 16 columns.
+template <class Row>
+__device__ __forceinline__ void dx_cols(uint32_t taddr, int cbeg, int cw, const Row& row, uint8_t* S2, int NT, int r,
+                                        const uint16_t* mask_in, int64_t stride, float sc, float* red) {
+  const int lane = threadIdx.x & 31;
+  for (int c = cbeg; c < cbeg + cw; c += 16) {
+    uint32_t v[16];
+    tmem_ld16x(taddr + (uint32_t)c, v);
+    tmem_wait_ld();
+    const uint32_t bits = mask_in[(int64_t)(c >> 4) * stride];
+    float dz[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) dz[u] = ((bits >> u) & 1u) ? __uint_as_float(v[u]) * sc : 0.0f;
+    uint32_t w[8];
+#pragma unroll
+    for (int h = 0; h < 8; ++h) w[h] = pack2(dz[2 * h], dz[2 * h + 1]);
+    row(r, c, w);
+    store_col16p(S2, NT, r, c, w);
+    const float sb = col_reduce16(dz);
+    if (lane < 16) red[c + lane] = sb;
+  }
+}
+
+// The width-1 output layer behind the last hidden one.
+struct OutLayer {
+  const float* bL;
+  const float* y;
+  int batch;
+  float* partWL;
+  float* partBL;
+  float* partLoss;
+  float* colpart;
+};
+
+// The row dots of a tile's n_split column parts (the ranks of a cluster,
+// PAIR_ONLY: at most two), added in rank order, by every thread of every rank's
+// epilogue, also after a timed-out wait (ok false): the total of row threadIdx.x.
+template <bool PAIR_ONLY>
+struct DsmemTotals {
+  int n_split;
+  __device__ __forceinline__ void sync() const { __syncthreads(); }
+  __device__ __forceinline__ float total(bool& ok, const EpiSmem& E) const {
+    const int tid = threadIdx.x;
+    if (n_split > 1) cluster_sync();
+    else __syncthreads();
+    float tot = 0.0f;
+    if (ok && tid < kM) {
+      tot = E.rowdot[tid];
+      if (n_split > 1) {
+        if (PAIR_ONLY || n_split == 2) {
+          const uint32_t me = cluster_ctarank();
+          const float other = ld_dsmem_f32(E.rowdot + tid, me ^ 1u);
+          tot = me == 0 ? tot + other : other + tot;
+        } else {  // four
+          float v[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) v[k] = ld_dsmem_f32(E.rowdot + tid, (uint32_t)k);
+          tot = ((v[0] + v[1]) + v[2]) + v[3];
+        }
+      }
+    }
+    return tot;
+  }
+  // the other ranks have read this CTA's row dots, and its yrow is complete
+  __device__ __forceinline__ void settle(bool&) const {
+    if (n_split > 1) cluster_sync();
+    else __syncthreads();
+  }
+};
+
+// The same for a cluster of two (or one CTA), each rank sending its row dots
+// to the other, counted on its barrier (armed before the kernel's first
+// cluster barrier), by the 512 threads of the epilogue.
+struct SentTotals {
+  float* other;  // [128]
+  uint64_t* bar;
+  int rank, CL;
+  __device__ __forceinline__ void sync() const { named_bar_sync(1, kT); }
+  __device__ __forceinline__ float total(bool& ok, const EpiSmem& E) const {
+    const int tid = threadIdx.x;
+    float tot = 0.0f;
+    if (ok && tid < kM) {
+      tot = E.rowdot[tid];  // (this thread's own store)
+      if (CL > 1) {
+        const uint32_t to = (uint32_t)rank ^ 1u;
+        st_async_f32(map_cluster(other + tid, to), tot, map_cluster(bar, to));
+        if (mbar_wait_cl(bar, 0)) tot = rank == 0 ? tot + other[tid] : other[tid] + tot;
+        else ok = false;
+      }
+    }
+    return tot;
+  }
+  __device__ __forceinline__ void settle(bool& ok) const { ok = named_bar_and(1, kT, ok); }
+};
+
+// Epilogue of the last hidden layer's columns [n0, n0 + NT) of a 128-row tile
+// by the whole CTA: output layer, loss, its gradients and dz.
+template <class Totals, class Row>
+__device__ __forceinline__ void out_epilogue(bool& ok, const OutLayer& o, uint32_t taddr, int NT, int N, int n0, int mt,
+                                             int m0, int ns, const Totals& totals, const Row& row, uint8_t* S2,
+                                             const EpiSmem& E) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int q = warp & 3, cq = warp >> 2;
+  const int r = 32 * q + lane, j = m0 + r;
+  const int cw = NT / 4, cbeg = cq * cw;
+  // pass 1: activations and this warp's part of the output dot product.  With
+  // all of 128 or 256 columns in one CTA, each warp keeps its two halves apart
+  // and the row dot is added as two CTAs of half the columns add it: the same
+  // order, the same bits.
+  const bool whole = NT == N && (NT == 128 || NT == 256);
+  if (ok) {
+    float dot = 0.0f, first = 0.0f;  // (two names: an indexed pair would live in local memory)
+    for (int c = cbeg; c < cbeg + cw; c += 16) {
+      if (whole && c == cbeg + cw / 2) {
+        first = dot;
+        dot = 0.0f;
+      }
+      uint32_t v[16];
+      tmem_ld16x(taddr + (uint32_t)c, v);
+      tmem_wait_ld();
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        const float4 b4 = reinterpret_cast<const float4*>(E.s_bias + c)[g];
+        const float4 w4 = reinterpret_cast<const float4*>(E.s_w + c)[g];
+        const float b[4] = {b4.x, b4.y, b4.z, b4.w}, wv[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float z = __uint_as_float(v[4 * g + e]) + b[e];
+          dot = fmaf(round_bf16(z > 0.0f ? z : 0.0f), wv[e], dot);
+        }
+      }
+    }
+    if (whole) {
+      E.rowq[(2 * cq) * 128 + r] = first;
+      E.rowq[(2 * cq + 1) * 128 + r] = dot;
+    } else {
+      E.rowq[cq * 128 + r] = dot;
+    }
+  }
+  totals.sync();
+  if (ok && tid < kM) {
+    const float lo = ((E.rowq[tid] + E.rowq[128 + tid]) + E.rowq[256 + tid]) + E.rowq[384 + tid];
+    E.rowdot[tid] =
+        whole ? lo + (((E.rowq[512 + tid] + E.rowq[640 + tid]) + E.rowq[768 + tid]) + E.rowq[896 + tid]) : lo;
+  }
+  const float tot = totals.total(ok, E);
+  if (ok && tid < kM) E.yrow[tid] = tot + __ldg(o.bL);
+  totals.settle(ok);
+  if (ok) {
+    const bool valid = j < o.batch;
+    const float yhat = E.yrow[r];
+    const float e = valid ? yhat - __ldg(o.y + j) : 0.0f;
+    const float dzL = valid ? 2.0f * e / (float)o.batch : 0.0f;
+    const float rd = round_bf16(dzL);
+    if (ns == 0 && cq == 0) {
+      float e2 = e * e, dsum = dzL;
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        e2 += __shfl_xor_sync(0xffffffffu, e2, o);
+        dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
+      }
+      if (lane == 0) {
+        E.wsum[q] = e2;
+        E.wsum[4 + q] = dsum;
+      }
+    }
+    // pass 2 (Z re-read from TMEM, so [Z > 0] is the same test as in pass 1):
+    // dW_L partial (sum_j bf16(dz_L[j]) a[j, c]) and dz = bf16(dz_L) bf16(w_L) [Z > 0]
+    for (int c = cbeg; c < cbeg + cw; c += 16) {
+      uint32_t v[16];
+      tmem_ld16x(taddr + (uint32_t)c, v);
+      tmem_wait_ld();
+      float pw[16], dz[16];
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        const float4 b4 = reinterpret_cast<const float4*>(E.s_bias + c)[g];
+        const float4 w4 = reinterpret_cast<const float4*>(E.s_w + c)[g];
+        const float b[4] = {b4.x, b4.y, b4.z, b4.w}, wv[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float z = __uint_as_float(v[4 * g + e]) + b[e];
+          const bool pos = z > 0.0f;
+          pw[4 * g + e] = rd * round_bf16(pos ? z : 0.0f);
+          dz[4 * g + e] = pos ? rd * wv[e] : 0.0f;
+        }
+      }
+      uint32_t w[8];
+#pragma unroll
+      for (int h = 0; h < 8; ++h) w[h] = pack2(dz[2 * h], dz[2 * h + 1]);
+      row(r, c, w);
+      store_col16p(S2, NT, r, c, w);
+      const float sw = col_reduce16(pw);
+      if (lane < 16) E.red2[q * 256 + c + lane] = sw;
+      const float sb = col_reduce16(dz);
+      if (lane < 16) E.red[q * 256 + c + lane] = sb;
+    }
+  }
+  totals.sync();
+  if (ok) {
+    for (int c = tid; c < NT; c += kT) {
+      o.partWL[(int64_t)mt * N + n0 + c] = col_total(E.red2, c);
+      o.colpart[(int64_t)mt * N + n0 + c] = col_total(E.red, c);
+    }
+    if (ns == 0 && tid == 0) {
+      o.partLoss[mt] = ((E.wsum[0] + E.wsum[1]) + E.wsum[2]) + E.wsum[3];
+      o.partBL[mt] = ((E.wsum[4] + E.wsum[5]) + E.wsum[6]) + E.wsum[7];
     }
   }
 }
@@ -297,14 +561,7 @@ __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* sm
   uint64_t* full = reinterpret_cast<uint64_t*>(tail);           // [kMaxChunks]
   uint64_t* done = full + kMaxChunks;
   uint64_t* used = done + 1;                                    // [kMaxChunks] K-block read by the products
-  float* s_bias = reinterpret_cast<float*>(tail + kTailBar);    // [256]
-  float* s_w = s_bias + 256;                                    // [256] bf16-rounded output weights
-  float* red = s_w + 256;                                       // [4][256] column sums by lane quadrant
-  float* red2 = red + 4 * 256;                                  // [4][256]
-  float* rowq = red2 + 4 * 256;                                 // [8][128] row dots by column group
-  float* rowdot = rowq + 8 * 128;                               // [128] this CTA's row dots
-  float* yrow = rowdot + 128;                                   // [128] predictions
-  float* wsum = yrow + 128;                                     // [8] warp partials
+  const EpiSmem E(tail + kTailBar);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int S = RING ? J.stages : kMaxChunks;
@@ -383,135 +640,19 @@ __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* sm
     }
     uint16_t* mask_out = J.mask_out + j + (int64_t)(n0 >> 4) * J.rows_pad;
     const bool drop = J.drop_h > 0;
-    fwd_cols<EMB>(tmem + lane_addr, s_bias, cbeg, cw, S1, S2, NT, r, mask_out, J.rows_pad, drop, h1,
+    fwd_cols<EMB>(tmem + lane_addr, E.s_bias, cbeg, cw, OwnRow{S1}, S2, NT, r, mask_out, J.rows_pad, drop, h1,
              ((uint64_t)j << 20) | (uint64_t)n0, args.drop_thr, args.drop_scale);
   } else if (ok && J.epi == TE_DX) {
-    for (int c = cbeg; c < cbeg + cw; c += 16) {
-      uint32_t v[16];
-      tmem_ld16x(tmem + lane_addr + (uint32_t)c, v);
-      tmem_wait_ld();
-      const uint32_t bits = J.mask_in[(int64_t)((n0 + c) >> 4) * J.rows_pad + j];
-      float dz[16];
-      const float sc = J.drop_h > 0 ? args.drop_scale : 1.0f;
-#pragma unroll
-      for (int u = 0; u < 16; ++u) dz[u] = ((bits >> u) & 1u) ? __uint_as_float(v[u]) * sc : 0.0f;
-      uint32_t w[8];
-#pragma unroll
-      for (int h = 0; h < 8; ++h) w[h] = pack2(dz[2 * h], dz[2 * h + 1]);
-      if (J.out) store_row16p(S1, kM, r, c, w);
-      store_col16p(S2, NT, r, c, w);
-      const float sb = col_reduce16(dz);
-      if (lane < 16) red[q * 256 + c + lane] = sb;
-    }
+    dx_cols(tmem + lane_addr, cbeg, cw, OwnRow{J.out ? S1 : nullptr}, S2, NT, r, J.mask_in + (int64_t)(n0 >> 4) * J.rows_pad + j,
+            J.rows_pad, J.drop_h > 0 ? args.drop_scale : 1.0f, E.red + q * 256);
     __syncthreads();
     for (int c = tid; c < NT; c += kT)
-      J.colpart[(int64_t)mt * N + n0 + c] = ((red[c] + red[256 + c]) + red[512 + c]) + red[768 + c];
+      J.colpart[(int64_t)mt * N + n0 + c] = col_total(E.red, c);
   }
   if (!EMB && J.epi == TE_FWD_OUT) {
-    // pass 1: activations and this warp's part of the output dot product
-    // With all 256 columns in one CTA (no cluster), each warp keeps its two
-    // 32-column halves apart and the row dot is added as the two 128-column
-    // CTAs of the cluster form add it: the same order, the same bits.
-    const bool whole = NT == 256;
-    if (ok) {
-      float dot[2] = {0.0f, 0.0f};
-      for (int c = cbeg; c < cbeg + cw; c += 16) {
-        uint32_t v[16];
-        tmem_ld16x(tmem + lane_addr + (uint32_t)c, v);
-        tmem_wait_ld();
-        const int hh = whole && c >= cbeg + 32 ? 1 : 0;
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-          const float z = __uint_as_float(v[u]) + s_bias[c + u];
-          dot[hh] = fmaf(round_bf16(z > 0.0f ? z : 0.0f), s_w[c + u], dot[hh]);
-        }
-      }
-      if (whole) {
-        rowq[(2 * cq) * 128 + r] = dot[0];
-        rowq[(2 * cq + 1) * 128 + r] = dot[1];
-      } else {
-        rowq[cq * 128 + r] = dot[0];
-      }
-    }
-    __syncthreads();
-    if (ok && tid < kM) {
-      const float lo = ((rowq[tid] + rowq[128 + tid]) + rowq[256 + tid]) + rowq[384 + tid];
-      rowdot[tid] = whole ? lo + (((rowq[512 + tid] + rowq[640 + tid]) + rowq[768 + tid]) + rowq[896 + tid]) : lo;
-    }
-    if (J.n_split > 1) cluster_sync();
-    else __syncthreads();
-    if (ok && tid < kM) {
-      float tot = rowdot[tid];
-      if (J.n_split > 1) {  // the ranks' parts in rank order on every rank
-        if (!RING || J.n_split == 2) {
-          const uint32_t me = cluster_ctarank();
-          const float other = ld_dsmem_f32(rowdot + tid, me ^ 1u);
-          tot = me == 0 ? tot + other : other + tot;
-        } else {  // four
-          float v[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) v[k] = ld_dsmem_f32(rowdot + tid, (uint32_t)k);
-          tot = ((v[0] + v[1]) + v[2]) + v[3];
-        }
-      }
-      yrow[tid] = tot + __ldg(J.bL);
-    }
-    if (J.n_split > 1) cluster_sync();  // the other ranks have read this CTA's rowdot
-    else __syncthreads();
-    if (ok) {
-      const bool valid = j < J.batch;
-      const float yhat = yrow[r];
-      const float e = valid ? yhat - __ldg(J.y + j) : 0.0f;
-      const float dzL = valid ? 2.0f * e / (float)J.batch : 0.0f;
-      const float rd = round_bf16(dzL);
-      if (ns == 0 && cq == 0) {
-        float e2 = e * e, dsum = dzL;
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-          e2 += __shfl_xor_sync(0xffffffffu, e2, o);
-          dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
-        }
-        if (lane == 0) {
-          wsum[q] = e2;
-          wsum[4 + q] = dsum;
-        }
-      }
-      // pass 2 (Z re-read from TMEM, so [Z > 0] is the same test as in pass 1):
-      // dW_L partial (sum_j bf16(dz_L[j]) a[j, c]) and dz = bf16(dz_L) bf16(w_L) [Z > 0]
-      for (int c = cbeg; c < cbeg + cw; c += 16) {
-        uint32_t v[16];
-        tmem_ld16x(tmem + lane_addr + (uint32_t)c, v);
-        tmem_wait_ld();
-        float pw[16], dz[16];
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-          const float z = __uint_as_float(v[u]) + s_bias[c + u];
-          const bool pos = z > 0.0f;
-          pw[u] = rd * round_bf16(pos ? z : 0.0f);
-          dz[u] = pos ? rd * s_w[c + u] : 0.0f;
-        }
-        uint32_t w[8];
-#pragma unroll
-        for (int h = 0; h < 8; ++h) w[h] = pack2(dz[2 * h], dz[2 * h + 1]);
-        if (J.out) store_row16p(S1, kM, r, c, w);
-        store_col16p(S2, NT, r, c, w);
-        const float sw = col_reduce16(pw);
-        if (lane < 16) red2[q * 256 + c + lane] = sw;
-        const float sb = col_reduce16(dz);
-        if (lane < 16) red[q * 256 + c + lane] = sb;
-      }
-    }
-    __syncthreads();
-    if (ok) {
-      for (int c = tid; c < NT; c += kT) {
-        J.partWL[(int64_t)mt * N + n0 + c] = ((red2[c] + red2[256 + c]) + red2[512 + c]) + red2[768 + c];
-        J.colpart[(int64_t)mt * N + n0 + c] = ((red[c] + red[256 + c]) + red[512 + c]) + red[768 + c];
-      }
-      if (ns == 0 && tid == 0) {
-        J.partLoss[mt] = ((wsum[0] + wsum[1]) + wsum[2]) + wsum[3];
-        J.partBL[mt] = ((wsum[4] + wsum[5]) + wsum[6]) + wsum[7];
-      }
-    }
+    const OutLayer o{J.bL, J.y, J.batch, J.partWL, J.partBL, J.partLoss, J.colpart};
+    out_epilogue(ok, o, tmem + lane_addr, NT, N, n0, mt, m0, ns, DsmemTotals<!RING>{J.n_split},
+                 OwnRow{J.out ? S1 : nullptr}, S2, E);
   }
   if (ok && J.epi != TE_STORE) {
     fence_async_smem();  // staged tiles are read by the bulk copies (async proxy)
@@ -566,7 +707,7 @@ __global__ void __launch_bounds__(kT, 1) k_tr_gemm(const __grid_constant__ TrArg
   // The next product may start now: its CTAs take SMs this grid leaves idle
   // and run their own prologue while this one works.  Every kernel of the
   // step after the gather starts only after the gather has passed its wait
-  // (it lets its successor in at its end), so after the previous step's
+  // (it lets its successor in behind it), so after the previous step's
   // optimiser has completed: the weight images and the master read before
   // the wait below are final.
   if (!EMB) pdl_trigger();
@@ -583,6 +724,401 @@ __global__ void __launch_bounds__(kT, 1) k_tr_gemm(const __grid_constant__ TrArg
   // completion makes them visible to the next kernel
   tr_tile<RING, EMB>(args, (int)blockIdx.x, smem, tmem, 0, false, true);
   if (threadIdx.x < 32) tmem_dealloc(tmem, tcols);
+}
+
+// The forward pass and the input gradients of a step in one launch: one CTA,
+// or a cluster of two, per 128-row tile; CTA `rank` has columns [rank * NT,
+// ...) of every product.  The tile's activations (then gradients) stay in
+// shared memory as the next product's operand: the epilogue stores its columns
+// into both CTAs' copies, the other's counted on its barriers.  Two copies in
+// turn need no cluster barrier: a rank writes the operand of product p + 1
+// once its own product p is done, so after the other has finished product
+// p - 1, which read that copy last.  Weights stream through a ring of K-blocks
+// that is filled ahead across products by a warp of its own; another issues
+// the products; sixteen run the epilogues.  Global memory gets only what the
+// weight gradients read, the transposed images.  Same tiles, products and
+// order of every sum as a launch per product, so the same bits.
+//
+// Bound by the chain of a tile: per product of 256 columns about 2.6K cycles
+// from operand to accumulator and 4-5.5K of epilogue arithmetic and stores
+// (11K for the output layer's).  Before, each product was a launch of its own,
+// 5.5-8 us with its prologue, loads and tail.  A step (this, the gather, the
+// weight gradients and the optimiser; us, a launch per product -> now):
+//   128-256-256-256-1  batch 4096  49.8 -> 47.0     64-128-128-128-1  512  34.4 -> 28.1
+//   64-128-128-128-1   batch 4096, dropout  41.0 -> 35.2              8192  50.0 -> 34.2
+//   128-192-192-1      batch 8192  43.2 -> 38.2     128-256-256-1     8192  51.1 -> 39.0
+//   128-256-256-1      batch 4096  35.5 -> 35.4     16-64-1           256  16.2 -> 15.0
+constexpr int kMaxPhases = 2 * (LS_MAX_LAYERS - 1);
+constexpr int kMaxRing = 8;
+constexpr int kChainT = kT + 64;  // the epilogue's warps, the products' warp, the weights' warp
+constexpr int kSmemMax = 227 * 1024;
+constexpr int kChainBar = 384;  // barriers and the TMEM address, before the epilogue scratch
+
+struct ChainPhase {
+  int epi;             // TE_FWD, TE_FWD_OUT or TE_DX
+  int nk;              // K-blocks
+  int NT;              // columns per CTA
+  int feeds;           // the next product reads the result
+  const uint8_t* B;    // weight image, NT * CL rows
+  const float* bias;
+  uint8_t* outT;       // transposed image of the result, rT rows
+  int rT;
+  int drop_h;          // as TrJob's
+  uint16_t* mask;      // written by TE_FWD, read by TE_DX
+  float* colpart;
+};
+
+struct ChainArgs {
+  ChainPhase ph[kMaxPhases];
+  int n, CL;
+  int a_bytes;         // one copy of the operand tile
+  int stages, stage_bytes;
+  uint32_t tmem_cols;
+  const uint8_t* A0;   // image of the minibatch, R rows
+  int R;
+  const float* wL;
+  OutLayer out;        // (colpart from the phase)
+  int* err;
+  const DevState* st;
+  uint64_t drop_seed, drop_thr;
+  float drop_scale;
+};
+
+__global__ void __launch_bounds__(kChainT, 1) k_tr_chain(const __grid_constant__ ChainArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* A = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* ring = A + 2 * (size_t)a.a_bytes;
+  uint64_t* afull = reinterpret_cast<uint64_t*>(ring + (size_t)a.stages * a.stage_bytes);  // [2][kMaxChunks]
+  uint64_t* done = afull + 2 * kMaxChunks;  // a product's accumulator is complete
+  uint64_t* ready = done + 1;               // the epilogue's warps have written the next operand's columns
+  uint64_t* xbar = ready + 1;               // the other rank's row dots
+  uint64_t* bfull = xbar + 1;               // [kMaxRing]
+  uint64_t* bempty = bfull + kMaxRing;      // [kMaxRing]
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bempty + kMaxRing);
+  volatile int* gave_up = reinterpret_cast<volatile int*>(tmem_holder + 1);
+  const EpiSmem E(reinterpret_cast<uint8_t*>(afull) + kChainBar);
+  float* other = E.s_bias + EpiSmem::kFloats;  // [128] the other rank's row dots
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int CL = a.CL;
+  const int rank = CL > 1 ? (int)cluster_ctarank() : 0;
+  const int mt = (int)blockIdx.x / CL, m0 = mt * kM;
+
+  if (tid == 0) {
+    for (int c = 0; c < 2 * kMaxChunks; ++c) mbar_init(&afull[c], 1);
+    mbar_init(done, 1);
+    mbar_init(ready, kT / 32);
+    mbar_init(xbar, 1);
+    for (int c = 0; c < a.stages; ++c) {
+      mbar_init(&bfull[c], 1);
+      mbar_init(&bempty[c], 1);
+    }
+    *gave_up = 0;
+    fence_mbar_init();
+    if (CL > 1) mbar_arrive_expect_tx(xbar, kM * 4);
+  }
+  __syncwarp();
+  if (warp == 0) {
+    tmem_alloc(tmem_holder, a.tmem_cols);
+    tmem_relinquish();
+  }
+  pdl_trigger();
+  tc_fence_before();
+  __syncthreads();
+  if (CL > 1) cluster_sync();  // both ranks' barriers are ready for the other's stores
+  tc_fence_after();
+  const uint32_t tmem = *tmem_holder;
+
+  if (warp == kT / 32 + 1) {
+    // weights: every product's K-blocks in order through the ring (final
+    // before this kernel starts: see k_tr_gemm)
+    if (lane == 0) {
+      int st = 0, loaded = 0;
+      uint32_t par = 0;  // of the reuse a stage waits for
+      bool ok = true;
+      for (int p = 0; ok && p < a.n; ++p) {
+        const uint32_t bytes = (uint32_t)a.ph[p].NT * 128;
+        const uint8_t* src = a.ph[p].B + (size_t)rank * bytes;
+        for (int c = 0; c < a.ph[p].nk; ++c, src += (size_t)CL * bytes) {
+          if (loaded >= a.stages && (!mbar_wait(&bempty[st], par) || *gave_up)) { ok = false; break; }
+          mbar_arrive_expect_tx(&bfull[st], bytes);
+          bulk_g2s(ring + (size_t)st * a.stage_bytes, src, bytes, &bfull[st]);
+          ++loaded;
+          if (++st == a.stages) {
+            st = 0;
+            par = loaded > a.stages ? par ^ 1u : 0u;
+          }
+        }
+      }
+      if (!ok) {  // copies under way land in this CTA's shared memory: wait for them (bounded)
+        *gave_up = 1;
+        for (int u = loaded > a.stages ? loaded - a.stages : 0; u < loaded; ++u)
+          if (!mbar_wait(&bfull[u % a.stages], (uint32_t)(u / a.stages) & 1u)) break;
+      }
+    }
+  } else if (warp == kT / 32) {
+    // products
+    if (lane == 0) {
+      pdl_wait();  // the minibatch from the gather
+      int cs = 0;
+      uint32_t cpar = 0, apar = 0;
+      int own0 = 0, own1 = 0;  // K-blocks of the operand that this CTA writes itself
+      for (int c = 0; c < a.ph[0].nk; ++c) {
+        mbar_arrive_expect_tx(&afull[c], kM * 128);
+        bulk_g2s(A + (size_t)c * kM * 128, a.A0 + ((size_t)c * a.R + m0) * 128, kM * 128, &afull[c]);
+      }
+      bool ok = true;
+      for (int p = 0; p < a.n; ++p) {
+        const int nk = a.ph[p].nk, NT = a.ph[p].NT;
+        const int buf = p & 1;
+        const uint32_t sA = smem_u32(A) + (uint32_t)buf * a.a_bytes;
+        uint64_t* af = afull + buf * kMaxChunks;
+        const uint32_t idesc = idesc_bf16_f32(kM, NT);
+        if (p > 0 && !mbar_wait(ready, (uint32_t)(p - 1) & 1u)) ok = false;
+        if (*gave_up) ok = false;
+        tc_fence_after();
+        for (int c = 0; ok && c < nk; ++c) {
+          if (c < own0 || c >= own1) {
+            const uint32_t bit = (uint32_t)(buf * kMaxChunks + c);
+            if (!mbar_wait_cl(&af[c], (apar >> bit) & 1u)) ok = false;
+            apar ^= 1u << bit;
+            fence_async_smem();  // the other rank's stores, read by the products
+          }
+          if (ok && !mbar_wait(&bfull[cs], cpar)) ok = false;
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t sa = sA + (uint32_t)c * kM * 128, sb = smem_u32(ring) + (uint32_t)cs * a.stage_bytes;
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            umma_bf16(tmem, sdesc_sw128(sa + 32u * k), sdesc_sw128(sb + 32u * k), idesc, (c | k) ? 1u : 0u);
+          umma_commit(&bempty[cs]);
+          if (++cs == a.stages) {
+            cs = 0;
+            cpar ^= 1u;
+          }
+        }
+        if (!ok) *gave_up = 1;
+        umma_commit(done);
+        if (!ok) break;
+        // the next operand's blocks of the other rank
+        own0 = rank * (NT / 64);
+        own1 = own0 + NT / 64;
+        if (p + 1 < a.n)
+          for (int c = 0; c < a.ph[p + 1].nk; ++c)
+            if (c < own0 || c >= own1)
+              mbar_arrive_expect_tx(&afull[(buf ^ 1) * kMaxChunks + c], kM * 128);
+      }
+      if (!ok)  // the minibatch's copies (a rank that gave up sends nothing more)
+        for (int c = 0; c < a.ph[0].nk && !(apar >> c & 1u); ++c)
+          if (!mbar_wait(&afull[c], 0)) break;
+    }
+  } else {
+    // epilogues
+    const int q = warp & 3, cq = warp >> 2;
+    const int r = 32 * q + lane, j = m0 + r;
+    const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16);
+    pdl_wait();  // targets and the step counter
+    bool ok = true;
+    for (int p = 0; ok && p < a.n; ++p) {
+      const ChainPhase& P = a.ph[p];
+      const int NT = P.NT, n0 = rank * NT;
+      for (int t = tid; t < NT; t += kT) {
+        if (P.bias) E.s_bias[t] = __ldg(P.bias + n0 + t);
+        if (P.epi == TE_FWD_OUT) E.s_w[t] = round_bf16(__ldg(a.wL + n0 + t));
+      }
+      if (tid == 0) bulk_commit_wait_read();  // the last product's stores have read S2
+      __syncwarp();
+      if (!mbar_wait(done, (uint32_t)p & 1u)) ok = false;
+      ok = named_bar_and(1, kT, ok && !*gave_up);  // one decision for the whole CTA
+      if (!ok) break;
+      tc_fence_after();
+      const int cw = NT / 4, cbeg = cq * cw, own0 = n0 / 64;
+      uint8_t* S1 = A + (size_t)((p + 1) & 1) * a.a_bytes + (size_t)own0 * kM * 128;
+      uint64_t* sb = afull + ((p + 1) & 1) * kMaxChunks + own0;
+      const bool send = CL > 1 && P.feeds;
+      const ClusterRow row{P.feeds ? S1 : nullptr, send ? map_cluster(S1, (uint32_t)rank ^ 1u) : 0,
+                           send ? map_cluster(sb, (uint32_t)rank ^ 1u) : 0};
+      // the transposed tile for its bulk stores takes this CTA's own columns
+      // of the operand just read: the other rank writes none of them, and this
+      // one not before its next epilogue
+      uint8_t* S2 = A + (size_t)(p & 1) * a.a_bytes + (size_t)own0 * kM * 128;
+      uint16_t* mask = P.mask + j + (int64_t)(n0 >> 4) * a.R;
+      if (P.epi == TE_FWD) {
+        uint64_t h1 = 0;
+        const bool drop = P.drop_h > 0;
+        if (drop) {  // (as in tr_tile)
+          const uint64_t t = (uint64_t)(*reinterpret_cast<const volatile int64_t*>(&a.st->step) + 1);
+          h1 = bh::mix64(a.drop_seed ^ ((t << 16) | (uint64_t)P.drop_h));
+        }
+        fwd_cols<false>(taddr, E.s_bias, cbeg, cw, row, S2, NT, r, mask, a.R, drop, h1,
+                        ((uint64_t)j << 20) | (uint64_t)n0, a.drop_thr, a.drop_scale);
+      } else if (P.epi == TE_DX) {
+        dx_cols(taddr, cbeg, cw, row, S2, NT, r, mask, a.R, P.drop_h > 0 ? a.drop_scale : 1.0f, E.red + q * 256);
+      } else {
+        OutLayer o = a.out;
+        o.colpart = P.colpart;
+        out_epilogue(ok, o, taddr, NT, NT * CL, n0, mt, m0, rank, SentTotals{other, xbar, rank, CL}, row, S2, E);
+        if (!ok) break;
+      }
+      tc_fence_before();
+      fence_async_smem();  // the columns are read by products and bulk copies
+      __syncwarp();
+      if (lane == 0) mbar_arrive(ready);
+      named_bar_sync(1, kT);
+      if (tid == 0)
+        for (int h = 0; h < kM / 64; ++h)
+          bulk_s2g(P.outT + ((int64_t)(m0 / 64 + h) * P.rT + n0) * 128, S2 + (size_t)h * NT * 128, (uint32_t)NT * 128);
+      if (P.epi == TE_DX)
+        for (int c = tid; c < NT; c += kT) P.colpart[(int64_t)mt * NT * CL + n0 + c] = col_total(E.red, c);
+    }
+    if (tid == 0) {
+      bulk_commit_wait_read();
+      if (!ok) {
+        *gave_up = 1;
+        latch_error(a.err, LS_ERR_TIMEOUT);
+      }
+    }
+    tc_fence_before();
+  }
+  __syncwarp();
+  __syncthreads();
+  if (CL > 1) cluster_sync();  // no rank leaves while the other may still store to it
+  tc_fence_after();
+  if (warp == 0) tmem_dealloc(tmem, a.tmem_cols);
+}
+
+// The weight gradients of every hidden layer in one launch: dW_l = dz_l^T A_l
+// as 128-row tiles x column parts x splits of the batch (k_tr_gemm's TE_STORE
+// jobs: same tiles, splits and order, so the same bits), two CTAs an SM: bound
+// by the operand reads from L2 (25 MB for 128-256-256-256-1 at batch 4096),
+// which one launch of all layers keeps going where one launch a layer left
+// half the SMs idle.
+struct DwJob {
+  const uint8_t* A;   // img(dz_l^T), rA rows
+  const uint8_t* B;   // img(A_l^T), NT * n_split rows
+  float* C;           // [split][M][ldc]
+  int rA, M, ldc;
+  int NT, n_split, m_tiles;
+  int nchunks, kblocks, stages;
+};
+constexpr int kDwT = 256;
+constexpr int kDwStage = 98304;  // operand stages: three of a 128-row and a 128-column K-block
+
+struct DwArgs {
+  DwJob job[LS_MAX_LAYERS - 1];
+  int cta0[LS_MAX_LAYERS];  // first CTA of each job
+  int n;
+  int* err;
+};
+
+__global__ void __launch_bounds__(kDwT, 2) k_tr_dw(const __grid_constant__ DwArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kDwStage);  // [kMaxRing]
+  uint64_t* empty = full + kMaxRing;                              // [kMaxRing]
+  uint64_t* done = empty + kMaxRing;
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(done + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  int jb = 0;
+#pragma unroll
+  for (int k = 1; k < LS_MAX_LAYERS - 1; ++k) jb += (k < a.n && (int)blockIdx.x >= a.cta0[k]) ? 1 : 0;
+  const DwJob& J = a.job[jb];
+  const int li = (int)blockIdx.x - a.cta0[jb];
+  const int ns = li % J.n_split, rest = li / J.n_split;
+  const int mt = rest % J.m_tiles, split = rest / J.m_tiles;
+  const int NT = J.NT, N = NT * J.n_split, n0 = ns * NT, m0 = mt * kM;
+  const int nch = min(J.nchunks, J.kblocks - split * J.nchunks), S = J.stages;
+  const uint32_t b_bytes = (uint32_t)NT * 128, stage_bytes = kM * 128 + b_bytes;
+  uint32_t tcols = 32;
+  while ((int)tcols < NT) tcols <<= 1;
+  if (tid == 0) {
+    for (int c = 0; c < S; ++c) {
+      mbar_init(&full[c], 1);
+      mbar_init(&empty[c], 1);
+    }
+    mbar_init(done, 1);
+    fence_mbar_init();
+  }
+  __syncwarp();
+  if (warp == 0) {
+    tmem_alloc(tmem_holder, tcols);
+    tmem_relinquish();
+  }
+  pdl_trigger();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_holder;
+  pdl_wait();  // the transposed images
+  bool ok = true;
+  if (tid == 0) {
+    auto load = [&](int c, int st) {
+      const size_t kb = (size_t)(split * J.nchunks + c);
+      uint8_t* to = smem + (size_t)st * stage_bytes;
+      mbar_arrive_expect_tx(&full[st], stage_bytes);
+      bulk_g2s(to, J.A + (kb * J.rA + m0) * 128, kM * 128, &full[st]);
+      bulk_g2s(to + kM * 128, J.B + (kb * N + n0) * 128, b_bytes, &full[st]);
+    };
+    int loaded = 0, st = 0, lst = 0;
+    uint32_t par = 0, lpar = 0;
+    for (; loaded < nch && loaded < S; ++loaded) load(loaded, loaded);
+    const uint32_t idesc = idesc_bf16_f32(kM, NT);
+    int c = 0;
+    for (; c < nch; ++c) {
+      if (!mbar_wait(&full[st], par)) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t sa = smem_u32(smem + (size_t)st * stage_bytes), sb = sa + kM * 128;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        umma_bf16(tmem, sdesc_sw128(sa + 32u * k), sdesc_sw128(sb + 32u * k), idesc, (c | k) ? 1u : 0u);
+      umma_commit(&empty[st]);
+      if (++st == S) {
+        st = 0;
+        par ^= 1u;
+      }
+      if (c > 0 && loaded < nch) {  // the previous K-block's stage
+        if (!mbar_wait(&empty[lst], lpar)) { ok = false; break; }
+        load(loaded, lst);
+        ++loaded;
+        if (++lst == S) {
+          lst = 0;
+          lpar ^= 1u;
+        }
+      }
+    }
+    if (!ok)  // copies under way land in this CTA's shared memory: wait for them (bounded)
+      for (; c < loaded; ++c) {
+        if (!mbar_wait(&full[st], par)) break;
+        if (++st == S) {
+          st = 0;
+          par ^= 1u;
+        }
+      }
+    umma_commit(done);
+  }
+  __syncwarp();
+  if (!mbar_wait(done, 0)) ok = false;
+  ok = __syncthreads_and(ok) != 0;
+  if (!ok) latch_error(a.err, LS_ERR_TIMEOUT);
+  tc_fence_after();
+  const int q = warp & 3, r = m0 + 32 * q + lane;
+  if (ok && r < J.M) {
+    const int cw = NT / 2, cbeg = (warp >> 2) * cw;
+    float* crow = J.C + ((int64_t)split * J.M + r) * J.ldc + n0;
+    const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16);
+    for (int c = cbeg; c < cbeg + cw; c += 16) {
+      uint32_t v[16];
+      tmem_ld16x(taddr + (uint32_t)c, v);
+      tmem_wait_ld();
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+        reinterpret_cast<float4*>(crow + c)[g] =
+            make_float4(__uint_as_float(v[4 * g]), __uint_as_float(v[4 * g + 1]), __uint_as_float(v[4 * g + 2]),
+                        __uint_as_float(v[4 * g + 3]));
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, tcols);
 }
 
 // Minibatch gather: row j of the batch (slot idx[j], or (step*B + j) mod
@@ -688,9 +1224,9 @@ __device__ __forceinline__ void tr_gather_items(const GatherArgs& g, int64_t fir
 
 __global__ void k_tr_gather(const __grid_constant__ GatherArgs g) {
   pdl_wait();  // the ring and the device counters from the previous kernels of the stream
+  pdl_trigger();
   tr_gather_items(g, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x,
                   blockIdx.x == 0 && threadIdx.x == 0);
-  pdl_trigger();
 }
 
 // sum_{s < n} src[s * stride], added in order, sixteen loads in flight.
@@ -857,7 +1393,6 @@ __global__ void __launch_bounds__(256) k_tr_opt(const __grid_constant__ OptArgs 
 // grid barrier between phases.  Same tiles, same epilogues and same order of
 // every sum as the launch-per-phase path, so the same bits.
 // ---------------------------------------------------------------------------
-constexpr int kMaxPhases = 2 * (LS_MAX_LAYERS - 1);
 constexpr uint32_t kGridSpin = 1u << 21;  // barrier polls before giving up (a second or so)
 
 struct StepArgs {
@@ -960,7 +1495,7 @@ __global__ void __launch_bounds__(kT, 1) k_tr_step(const __grid_constant__ StepA
 }
 
 int gemm_smem_bytes() {
-  return 1024 + kStageRegion + kTailBar + (256 + 256 + 8 * 256 + 8 * 128 + 128 + 128 + 8) * 4;
+  return 1024 + kStageRegion + kTailBar + EpiSmem::kFloats * 4;
 }
 
 TrArgs tr_args(const Ctx& c, const TrJob& j0, const TrJob* j1, int* err) {
@@ -1021,6 +1556,46 @@ int n_split_out(int N) { return N == 512 ? 4 : N > 256 ? 2 : n_split_for(N); }
 
 }  // namespace
 
+namespace {
+
+// Shape of the one-launch forward and input-gradient pass (k_tr_chain); CL 0:
+// a launch per product.  The CTAs of a tile's cluster are the column parts of
+// the output product, so that the row dot products add up in the same order;
+// every hidden layer has to split into as many parts of whole K-blocks, and
+// two copies of the operand tile and three K-blocks of weights have to fit:
+// layers up to 256.  (With one copy and a cluster barrier per product, layers
+// of 512 in clusters of four came out even at batch 4096, 55.7 us against
+// 56.1, and behind at 256, 45.5 against 40.7: a rank's 32 KB for each of three
+// others pass at some 11 bytes a cycle.)  Layers of up to 128 columns stay
+// whole once two CTAs a tile would not all be resident: 34.2 us either way at
+// batch 8192 of 64-128-128-128-1, 39.4 against 35.2 with dropout at 4096.
+struct ChainPlan {
+  int CL = 0, a_bytes = 0, stages = 0, stage_bytes = 0, nt_max = 0, smem = 0;
+};
+ChainPlan plan_chain(const MlpDesc& m, const TrainFast& f, int T, int sms) {
+  ChainPlan p;
+  const int nh = m.n_layers - 1;
+  int w_max = 0;
+  for (int l = 1; l <= nh; ++l) w_max = std::max(w_max, m.w[l]);
+  const int parts = n_split_out(m.w[nh]);
+  const int CL = w_max <= 128 && T * parts > sms ? 1 : parts;
+  if (CL > 2) return p;
+  for (int l = 1; l <= nh; ++l) {
+    if (m.w[l] % (64 * CL) != 0 || m.w[l] / CL > 256) return p;
+    p.nt_max = std::max(p.nt_max, m.w[l] / CL);
+  }
+  p.a_bytes = kM * std::max(f.in_pad[0], w_max) * 2;
+  p.stage_bytes = p.nt_max * 128;
+  const int fixed = 1024 + 2 * p.a_bytes + kChainBar + (EpiSmem::kFloats + kM) * 4;
+  p.stages = std::min(kMaxRing, (kSmemMax - fixed) / p.stage_bytes);
+  if (p.stages < 3) return p;
+  p.smem = fixed + p.stages * p.stage_bytes;
+  p.CL = CL;
+  return p;
+}
+
+}  // namespace
+
 // The fast path applies to bf16 predictors with at least one hidden layer,
 // hidden widths that are multiples of 64 up to 256, or 384 or 512, and an
 // input width of at most 256 (padded to 64).  Layers wider than 256 stream
@@ -1042,7 +1617,14 @@ bool plan_train_fast(const MlpDesc& m, int max_batch, TrainFast& f) {
   }
   f.rows_max = ((max_batch + kM - 1) / kM) * kM;
   f.on = true;
+  f.chain = plan_chain(m, f, 1, 152).CL;
   return true;
+}
+
+// dz^T images: one a layer where the weight gradients run after the whole
+// backward pass, else two by layer parity.
+static int train_dzt_images(const MlpDesc& m, const TrainFast& f) {
+  return f.chain ? std::max(2, m.n_layers - 1) : 2;
 }
 
 int64_t train_fast_bytes(const MlpDesc& m, const TrainFast& f, int64_t* parts_floats) {
@@ -1053,7 +1635,7 @@ int64_t train_fast_bytes(const MlpDesc& m, const TrainFast& f, int64_t* parts_fl
   int hmax = 0;
   for (int l = 1; l <= nh; ++l) hmax = std::max(hmax, m.w[l]);
   const int64_t hpad = ((hmax + 127) / 128) * 128;
-  bytes += 2 * (R * hmax * 2 + hpad * R * 2);                       // dz images, two parities
+  bytes += 2 * R * hmax * 2 + train_dzt_images(m, f) * hpad * R * 2;  // dz images and transposes
   for (int l = 1; l <= nh; ++l) bytes += (int64_t)(m.w[l] / 32) * R * 4;  // masks
   for (int l = 0; l < nh; ++l) bytes += 2 * (int64_t)m.w[l + 1] * f.in_pad[l] * 2;  // weight images
   const int64_t T = R / kM;
@@ -1081,6 +1663,8 @@ void train_fast_bind(const MlpDesc& m, TrainFast& f, uint8_t* base, float* parts
   for (int b = 0; b < 2; ++b) {
     f.imgDZ[b] = p;
     p += R * hmax * 2;
+  }
+  for (int b = 0; b < train_dzt_images(m, f); ++b) {
     f.imgDZT[b] = p;
     p += hpad * R * 2;
   }
@@ -1173,6 +1757,26 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
   const int T = R / kM;
   // one persistent launch (the products become its phases) or one launch each
   const bool one = c.train_ctas > 0;
+  const bool chain = !one && f.chain > 0;
+  const ChainPlan cp = chain ? plan_chain(m, f, T, c.sms) : ChainPlan{};
+  ChainArgs ca{};
+  DwArgs da{};
+  int dw_ctas = 0;
+  auto chain_phase = [&](const TrJob& J, int K, bool feeds) {
+    ChainPhase& P = ca.ph[ca.n++];
+    P.epi = J.epi;
+    P.nk = K / 64;
+    P.NT = J.NT * J.n_split / cp.CL;
+    P.feeds = feeds;
+    P.B = J.B;
+    P.bias = J.bias;
+    P.outT = J.outT;
+    P.rT = J.rT;
+    P.drop_h = J.drop_h;
+    P.mask = J.epi == TE_DX ? const_cast<uint16_t*>(J.mask_in) : J.mask_out;
+    P.colpart = J.colpart;
+  };
+  const auto dzt = [&](int l) { return f.imgDZT[chain ? l : l & 1]; };
   static thread_local StepArgs step;
   step = StepArgs{};
   cudaError_t e = cudaSuccess;
@@ -1210,7 +1814,7 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
       J.mask_out = f.mask[l + 1];
     } else {
       J.out = l > 0 ? f.imgDZ[l & 1] : nullptr;
-      J.outT = f.imgDZT[l & 1];
+      J.outT = dzt(l);
       J.rT = ((m.w[l + 1] + 127) / 128) * 128;
       J.colpart = f.partB[l];
       J.wL = c.master + m.woff[nh];
@@ -1225,6 +1829,11 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
     J.drop_h = (c.cfg.dropout > 0.0f && l + 2 < m.n_layers) ? l + 1 : 0;
     if (one) {
       step.ph[step.n_ph++] = tr_args(c, J, nullptr, c.d_err);
+      continue;
+    }
+    if (chain) {
+      chain_phase(J, f.in_pad[l], !last || nh > 1);
+      if (last) ca.out = OutLayer{J.bL, J.y, J.batch, J.partWL, J.partBL, J.partLoss, nullptr};
       continue;
     }
     e = traced(c, TR_GEMM_TC_FWD, 1, s, [&] { return launch_tr_gemm(c, J, nullptr, c.d_err, s); });
@@ -1246,7 +1855,7 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
     W.nchunks = std::min(kpc, W.kblocks);
     W.splits = (W.kblocks + W.nchunks - 1) / W.nchunks;  // the last one may be short
     W.NT = f.in_pad[l] / W.n_split;
-    W.A = f.imgDZT[l & 1];
+    W.A = dzt(l);
     W.rA = ((out + 127) / 128) * 128;
     W.B = f.imgAT[l];
     W.M = out;
@@ -1269,7 +1878,7 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
       X.rows_pad = R;
       X.mask_in = f.mask[l];
       X.out = l > 1 ? f.imgDZ[(l - 1) & 1] : nullptr;
-      X.outT = f.imgDZT[(l - 1) & 1];
+      X.outT = dzt(l - 1);
       X.rT = ((m.w[l] + 127) / 128) * 128;
       X.colpart = f.partB[l - 1];
       X.drop_h = (c.cfg.dropout > 0.0f && l < m.n_layers - 1) ? l : 0;  // input a_l was dropped
@@ -1278,8 +1887,48 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
       step.ph[step.n_ph++] = tr_args(c, W, l > 0 ? &X : nullptr, c.d_err);
       continue;
     }
+    if (chain) {
+      if (l > 0) chain_phase(X, out, l > 1);
+      da.cta0[da.n] = dw_ctas;
+      DwJob& D = da.job[da.n++];
+      D = DwJob{W.A, W.B, W.C, W.rA, W.M, W.ldc, W.NT, W.n_split, W.m_tiles, W.nchunks, W.kblocks, 0};
+      D.stages = std::min({kMaxRing, W.nchunks, kDwStage / ((kM + W.NT) * 128)});
+      dw_ctas += W.m_tiles * W.n_split * W.splits;
+      continue;
+    }
     e = traced(c, l > 0 ? TR_GEMM_TC_DX : TR_GEMM_TC_DW, 1, s,
                [&] { return launch_tr_gemm(c, W, l > 0 ? &X : nullptr, c.d_err, s); });
+    if (e != cudaSuccess) return e;
+  }
+  if (chain) {
+    ca.CL = cp.CL;
+    ca.a_bytes = cp.a_bytes;
+    ca.stages = cp.stages;
+    ca.stage_bytes = cp.stage_bytes;
+    ca.tmem_cols = 32;
+    while ((int)ca.tmem_cols < cp.nt_max) ca.tmem_cols <<= 1;
+    ca.A0 = f.imgA[0];
+    ca.R = R;
+    ca.wL = c.master + m.woff[nh];
+    const TrArgs t = tr_args(c, TrJob{}, nullptr, c.d_err);  // (the dropout stream)
+    ca.err = t.err;
+    ca.st = t.st;
+    ca.drop_seed = t.drop_seed;
+    ca.drop_thr = t.drop_thr;
+    ca.drop_scale = t.drop_scale;
+    e = traced(c, TR_GEMM_TC_FWD, 1, s, [&] {
+      const cudaError_t e2 = cudaFuncSetAttribute(k_tr_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, cp.smem);
+      if (e2 != cudaSuccess) return e2;
+      return launch_chained(k_tr_chain, dim3(T * cp.CL), dim3(kChainT), (size_t)cp.smem, s, cp.CL, ca);
+    });
+    if (e != cudaSuccess) return e;
+    da.err = c.d_err;
+    e = traced(c, TR_GEMM_TC_DW, 1, s, [&] {
+      const int smem = 1024 + kDwStage + (2 * kMaxRing + 2) * 8;
+      const cudaError_t e2 = cudaFuncSetAttribute(k_tr_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (e2 != cudaSuccess) return e2;
+      return launch_chained(k_tr_dw, dim3(dw_ctas), dim3(kDwT), (size_t)smem, s, 1, da);
+    });
     if (e != cudaSuccess) return e;
   }
   OptArgs a{};

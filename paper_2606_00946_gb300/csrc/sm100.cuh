@@ -179,6 +179,25 @@ __device__ __forceinline__ float ld_dsmem_f32(const void* local, uint32_t rank) 
   return v;
 }
 
+// Shared-memory address of `local`'s offset in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t map_cluster(const void* local, uint32_t rank) {
+  uint32_t remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(local)), "r"(rank));
+  return remote;
+}
+// Stores into another CTA of the cluster, their bytes counted on its barrier
+// `bar` (both addresses from map_cluster).
+__device__ __forceinline__ void st_async_v4(uint32_t at, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(at),
+               "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void st_async_f32(uint32_t at, float v, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(at),
+               "r"(__float_as_uint(v)), "r"(bar)
+               : "memory");
+}
+
 // ---------------------------------------------------------------------------
 // packed arithmetic (two fp32 lanes in one 64-bit register; bf16x2)
 // ---------------------------------------------------------------------------
