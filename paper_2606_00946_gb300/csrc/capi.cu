@@ -314,6 +314,8 @@ int ls_create(const ls_config* cfg, ls_ctx** out) {
     if (e == cudaSuccess) train_fast_bind(m, c.tf, c.tf.base, c.tf.parts);
     c.train_ctas = cfg->train_ctas > 0 && !c.tf.wide ? std::min(cfg->train_ctas, c.sms) : 0;
   }
+  A(c.use_tc ? prepare_score_tc(c.tc) : prepare_score_simt());
+  if (fast_train) A(prepare_train_fast(c.tf));
   if (e == cudaSuccess) {
     A(cudaEventCreateWithFlags(&c.ev_pub, cudaEventDisableTiming));
     A(cudaEventCreateWithFlags(&c.ev_route, cudaEventDisableTiming));

@@ -404,6 +404,20 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// Lets `kernel` take all the dynamic shared memory that its static part leaves
+// of a CTA's 227 KB.  Called for a context's kernels when it is created: the
+// attribute call costs the host about as much as a tenth of a launch, so it is
+// kept out of the calls (every context sets the same value, so none shrinks
+// what another relies on).
+template <typename... KArgs>
+cudaError_t allow_smem(void (*kernel)(KArgs...)) {
+  cudaFuncAttributes fa{};
+  const cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              227 * 1024 - (int)fa.sharedSizeBytes);
+}
+
 // ---------------------------------------------------------------------------
 // launchers (each returns the launch status)
 // ---------------------------------------------------------------------------
@@ -489,6 +503,9 @@ inline bool scorer_selects(const TcPlan& p, int n_req, int n_inst) {
   if (p.pair || p.wide) return false;
   return (n_inst <= 128 && 128 % n_inst == 0) || (int64_t)n_req * n_inst <= 128;
 }
+cudaError_t prepare_score_tc(const TcPlan& p);  // once per context, before its first launch
+cudaError_t prepare_score_simt();
+cudaError_t prepare_train_fast(const TrainFast& f);
 cudaError_t launch_score_tc(const MlpDesc& m, const TcPlan& p, const Published* pub, const int32_t* sel,
                             int n_req, int n_inst, const uint4* pairx, const uint8_t* ximg, int32_t* choice,
                             float* best,

@@ -478,6 +478,13 @@ SimtPlan plan_simt(const MlpDesc& m, int n_req, int n_inst, int sms) {
 
 bool simt_selects(const MlpDesc& m, int n_req, int n_inst, int sms) { return plan_simt(m, n_req, n_inst, sms).rq > 0; }
 
+cudaError_t prepare_score_simt() {
+  cudaError_t e = allow_smem(k_score_simt<4, true>);
+  if (e == cudaSuccess) e = allow_smem(k_score_simt<4, false>);
+  if (e == cudaSuccess) e = allow_smem(k_score_simt<8, true>);
+  return e == cudaSuccess ? allow_smem(k_score_simt<8, false>) : e;
+}
+
 cudaError_t launch_score_simt(const MlpDesc& mlp, const Published* pub, const int32_t* sel, int n_req, int n_inst,
                               const int64_t* tok_off, const int32_t* hits, const float* inst_state,
                               int d_inst, const float* req_feats, int d_req, const float* mean,
@@ -510,8 +517,6 @@ cudaError_t launch_score_simt(const MlpDesc& mlp, const Published* pub, const in
   a.best = best;
   auto* k = p.tr <= 16 ? (p.staged ? k_score_simt<4, true> : k_score_simt<4, false>)
                        : (p.staged ? k_score_simt<8, true> : k_score_simt<8, false>);
-  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
-  if (e != cudaSuccess) return e;
   const int grid = (int)std::min<int64_t>(a.tiles, 2 * (int64_t)sms);
   return launch_chained(k, dim3(grid), dim3(kSimtT), (size_t)p.smem, s, 1, a);
 }

@@ -1524,8 +1524,6 @@ cudaError_t launch_tr_args(const Ctx& c, const TrArgs& a, bool emb, cudaStream_t
   const int smem = gemm_smem_bytes();
   auto* k = emb ? (c.tf.wide ? k_tr_gemm<true, true> : k_tr_gemm<false, true>)
                 : (c.tf.wide ? k_tr_gemm<true, false> : k_tr_gemm<false, false>);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
   // the column parts of a TE_FWD_OUT tile exchange row sums through
   // distributed shared memory: one cluster per tile
   const int cl = j0.epi == TE_FWD_OUT ? j0.n_split : 1;
@@ -1749,6 +1747,13 @@ GatherArgs gather_args(const Ctx& c, int B, const int32_t* idx) {
 }
 }  // namespace
 
+cudaError_t prepare_train_fast(const TrainFast& f) {
+  cudaError_t e = f.wide ? allow_smem(k_tr_gemm<true, false>) : allow_smem(k_tr_gemm<false, false>);
+  if (e == cudaSuccess) e = f.wide ? allow_smem(k_tr_gemm<true, true>) : allow_smem(k_tr_gemm<false, true>);
+  if (e == cudaSuccess) e = allow_smem(k_tr_chain);
+  return e == cudaSuccess ? allow_smem(k_tr_dw) : e;
+}
+
 cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr, float* loss_out, cudaStream_t s) {
   const MlpDesc& m = c.mlp;
   TrainFast& f = c.tf;
@@ -1917,16 +1922,12 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
     ca.drop_thr = t.drop_thr;
     ca.drop_scale = t.drop_scale;
     e = traced(c, TR_GEMM_TC_FWD, 1, s, [&] {
-      const cudaError_t e2 = cudaFuncSetAttribute(k_tr_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, cp.smem);
-      if (e2 != cudaSuccess) return e2;
       return launch_chained(k_tr_chain, dim3(T * cp.CL), dim3(kChainT), (size_t)cp.smem, s, cp.CL, ca);
     });
     if (e != cudaSuccess) return e;
     da.err = c.d_err;
     e = traced(c, TR_GEMM_TC_DW, 1, s, [&] {
       const int smem = 1024 + kDwStage + (2 * kMaxRing + 2) * 8;
-      const cudaError_t e2 = cudaFuncSetAttribute(k_tr_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (e2 != cudaSuccess) return e2;
       return launch_chained(k_tr_dw, dim3(dw_ctas), dim3(kDwT), (size_t)smem, s, 1, da);
     });
     if (e != cudaSuccess) return e;
