@@ -744,10 +744,10 @@ __global__ void __launch_bounds__(kT, 1) k_tr_gemm(const __grid_constant__ TrArg
 // (11K for the output layer's).  Before, each product was a launch of its own,
 // 5.5-8 us with its prologue, loads and tail.  A step (this, the gather, the
 // weight gradients and the optimiser; us, a launch per product -> now):
-//   128-256-256-256-1  batch 4096  49.8 -> 47.0     64-128-128-128-1  512  34.4 -> 28.1
-//   64-128-128-128-1   batch 4096, dropout  41.0 -> 35.2              8192  50.0 -> 34.2
-//   128-192-192-1      batch 8192  43.2 -> 38.2     128-256-256-1     8192  51.1 -> 39.0
-//   128-256-256-1      batch 4096  35.5 -> 35.4     16-64-1           256  16.2 -> 15.0
+//   128-256-256-256-1  batch 4096  49.8 -> 46.0     64-128-128-128-1  512  34.4 -> 25.8
+//   64-128-128-128-1   batch 4096, dropout  41.0 -> 34.1              8192  50.0 -> 34.0
+//   128-192-192-1      batch 8192  43.2 -> 37.2     128-256-256-1     8192  51.1 -> 37.7
+//   128-256-256-1      batch 4096  35.5 -> 34.7     16-64-1           256  16.2 -> 15.4
 constexpr int kMaxPhases = 2 * (LS_MAX_LAYERS - 1);
 constexpr int kMaxRing = 8;
 constexpr int kChainT = kT + 64;  // the epilogue's warps, the products' warp, the weights' warp
@@ -1565,8 +1565,9 @@ namespace {
 // of 512 in clusters of four came out even at batch 4096, 55.7 us against
 // 56.1, and behind at 256, 45.5 against 40.7: a rank's 32 KB for each of three
 // others pass at some 11 bytes a cycle.)  Layers of up to 128 columns stay
-// whole once two CTAs a tile would not all be resident: 34.2 us either way at
-// batch 8192 of 64-128-128-128-1, 39.4 against 35.2 with dropout at 4096.
+// whole once two CTAs a tile would not all be resident; while they are, two are
+// the better: 35.2 us against 39.4 at batch 4096 of 64-128-128-128-1 with
+// dropout.
 struct ChainPlan {
   int CL = 0, a_bytes = 0, stages = 0, stage_bytes = 0, nt_max = 0, smem = 0;
 };
