@@ -467,6 +467,34 @@ __device__ __forceinline__ void out_epilogue(bool& ok, const OutLayer& o, uint32
   }
 }
 
+// fp32 tile of a weight-gradient partial: the warp's 32 rows and columns
+// [cbeg, cbeg + cw) from TMEM into `tile` (rows of NT floats and 16 bytes more,
+// so that the rows of a quarter warp start in different banks).
+__device__ __forceinline__ void store_tile(uint32_t taddr, int r, int cbeg, int cw, int NT, uint8_t* tile) {
+  uint8_t* row = tile + (size_t)r * (NT * 4 + 16);
+  for (int c = cbeg; c < cbeg + cw; c += 16) {
+    uint32_t v[16];
+    tmem_ld16x(taddr + (uint32_t)c, v);
+    tmem_wait_ld();
+#pragma unroll
+    for (int g = 0; g < 4; ++g)
+      *reinterpret_cast<uint4*>(row + (c + 4 * g) * 4) = make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+  }
+}
+
+// The tile's valid rows to global memory (row pitch ldc floats), a bulk copy
+// each, by the first 128 threads once every warp has stored (and fenced).
+// Stores from the threads' registers touch 32 lines an instruction and took
+// the load-store unit 4K cycles a tile of 128 columns.
+__device__ __forceinline__ void copy_tile(float* C, int ldc, int rows, int NT, const uint8_t* tile, bool drain) {
+  const int r = threadIdx.x;
+  if (r < rows && r < kM) bulk_s2g(C + (int64_t)r * ldc, tile + (size_t)r * (NT * 4 + 16), (uint32_t)NT * 4);
+  if (r < kM) {
+    if (drain) bulk_commit_wait_all();  // (tr_tile)
+    else bulk_commit_wait_read();
+  }
+}
+
 // Shared memory of a training-product CTA: the operand stages, then the
 // barriers (kMaxChunks `full`, `done`, kMaxChunks `used`) and epilogue scratch.
 __device__ __forceinline__ uint8_t* tr_tail(uint8_t* smem) { return smem + kStageRegion; }
@@ -616,19 +644,10 @@ __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* sm
   const uint32_t lane_addr = (uint32_t)(32 * q) << 16;
 
   if (ok && J.epi == TE_STORE) {
-    if (j < J.M) {
-      float* crow = J.C + (int64_t)split * J.split_stride + (int64_t)j * J.ldc + n0;
-      for (int c = cbeg; c < cbeg + cw; c += 16) {
-        uint32_t v[16];
-        tmem_ld16x(tmem + lane_addr + (uint32_t)c, v);
-        tmem_wait_ld();
-#pragma unroll
-        for (int g = 0; g < 4; ++g)
-          reinterpret_cast<float4*>(crow + c)[g] =
-              make_float4(__uint_as_float(v[4 * g]), __uint_as_float(v[4 * g + 1]), __uint_as_float(v[4 * g + 2]),
-                          __uint_as_float(v[4 * g + 3]));
-      }
-    }
+    if (j < J.M) store_tile(tmem + lane_addr, r, cbeg, cw, NT, smem);
+    fence_async_smem();
+    __syncthreads();
+    copy_tile(J.C + (int64_t)split * J.split_stride + (int64_t)m0 * J.ldc + n0, J.ldc, J.M - m0, NT, smem, drain);
   } else if (ok && J.epi == TE_FWD) {
     // dropout stream of this activation at step t = step + 1 (Sec. 4.1: dropout
     // between hidden layers): h1 = mix64(seed ^ ((t << 16) | h)),
@@ -744,10 +763,12 @@ __global__ void __launch_bounds__(kT, 1) k_tr_gemm(const __grid_constant__ TrArg
 // (11K for the output layer's).  Before, each product was a launch of its own,
 // 5.5-8 us with its prologue, loads and tail.  A step (this, the gather, the
 // weight gradients and the optimiser; us, a launch per product -> now):
-//   128-256-256-256-1  batch 4096  49.8 -> 46.0     64-128-128-128-1  512  34.4 -> 25.8
-//   64-128-128-128-1   batch 4096, dropout  41.0 -> 34.1              8192  50.0 -> 34.0
-//   128-192-192-1      batch 8192  43.2 -> 37.2     128-256-256-1     8192  51.1 -> 37.7
-//   128-256-256-1      batch 4096  35.5 -> 34.7     16-64-1           256  16.2 -> 15.4
+//   128-256-256-256-1  batch 4096  49.8 -> 41.8     64-128-128-128-1  512  34.4 -> 25.9
+//   64-128-128-128-1   batch 4096, dropout  41.0 -> 32.8              8192  50.0 -> 32.8
+//   128-192-192-1      batch 8192  43.2 -> 34.0     128-256-256-1     8192  51.1 -> 34.5
+//   128-256-256-1      batch 4096  35.5 -> 31.2     16-64-1           256  16.2 -> 16.0
+// (of which the weight gradients' row copies, see copy_tile: 46.0 -> 41.8 for
+// the first, 37.2 -> 34.0 and 37.7 -> 34.5 for the third row).
 constexpr int kMaxPhases = 2 * (LS_MAX_LAYERS - 1);
 constexpr int kMaxRing = 8;
 constexpr int kChainT = kT + 64;  // the epilogue's warps, the products' warp, the weights' warp
@@ -1001,7 +1022,7 @@ struct DwJob {
   int nchunks, kblocks, stages;
 };
 constexpr int kDwT = 256;
-constexpr int kDwStage = 98304;  // operand stages: three of a 128-row and a 128-column K-block
+constexpr int kDwStage = kM * (192 * 4 + 16);  // operand stages, then the fp32 tile of at most 192 columns
 
 struct DwArgs {
   DwJob job[LS_MAX_LAYERS - 1];
@@ -1100,24 +1121,13 @@ __global__ void __launch_bounds__(kDwT, 2) k_tr_dw(const __grid_constant__ DwArg
   ok = __syncthreads_and(ok) != 0;
   if (!ok) latch_error(a.err, LS_ERR_TIMEOUT);
   tc_fence_after();
-  const int q = warp & 3, r = m0 + 32 * q + lane;
-  if (ok && r < J.M) {
-    const int cw = NT / 2, cbeg = (warp >> 2) * cw;
-    float* crow = J.C + ((int64_t)split * J.M + r) * J.ldc + n0;
-    const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16);
-    for (int c = cbeg; c < cbeg + cw; c += 16) {
-      uint32_t v[16];
-      tmem_ld16x(taddr + (uint32_t)c, v);
-      tmem_wait_ld();
-#pragma unroll
-      for (int g = 0; g < 4; ++g)
-        reinterpret_cast<float4*>(crow + c)[g] =
-            make_float4(__uint_as_float(v[4 * g]), __uint_as_float(v[4 * g + 1]), __uint_as_float(v[4 * g + 2]),
-                        __uint_as_float(v[4 * g + 3]));
-    }
-  }
+  const int q = warp & 3, r = 32 * q + lane;
+  if (ok && m0 + r < J.M) store_tile(tmem + ((uint32_t)(32 * q) << 16), r, (warp >> 2) * (NT / 2), NT / 2, NT, smem);
+  fence_async_smem();
   tc_fence_before();
   __syncthreads();
+  if (ok) copy_tile(J.C + ((int64_t)split * J.M + m0) * J.ldc + n0, J.ldc, J.M - m0, NT, smem, false);
+  __syncwarp();
   if (warp == 0) tmem_dealloc(tmem, tcols);
 }
 
