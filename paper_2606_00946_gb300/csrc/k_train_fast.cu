@@ -257,16 +257,19 @@ __device__ __forceinline__ float col_total(const float* red, int c) {
 
 // Input-gradient epilogue of one warp's columns: dz = acc [mask] sc, its
 // images (the row-major one through `row`) and the column sums of the 32 rows
-// into red.  mask_in: this row's 16-bit words, `stride` apart by 16 columns.
+// into red.  mask_in: this row's 16-bit words, `stride` apart by 16 columns;
+// `bits` the warp's first one, loaded by the caller before it waited for the
+// product (each later one is requested a step ahead).
 template <class Row>
 __device__ __forceinline__ void dx_cols(uint32_t taddr, int cbeg, int cw, const Row& row, uint8_t* S2, int NT, int r,
-                                        const uint16_t* mask_in, int64_t stride, float sc, float* red) {
+                                        const uint16_t* mask_in, int64_t stride, uint32_t bits, float sc,
+                                        float* red) {
   const int lane = threadIdx.x & 31;
   for (int c = cbeg; c < cbeg + cw; c += 16) {
     uint32_t v[16];
     tmem_ld16x(taddr + (uint32_t)c, v);
     tmem_wait_ld();
-    const uint32_t bits = mask_in[(int64_t)(c >> 4) * stride];
+    const uint32_t next = c + 16 < cbeg + cw ? mask_in[(int64_t)((c >> 4) + 1) * stride] : 0u;
     float dz[16];
 #pragma unroll
     for (int u = 0; u < 16; ++u) dz[u] = ((bits >> u) & 1u) ? __uint_as_float(v[u]) * sc : 0.0f;
@@ -277,6 +280,7 @@ __device__ __forceinline__ void dx_cols(uint32_t taddr, int cbeg, int cw, const 
     store_col16p(S2, NT, r, c, w);
     const float sb = col_reduce16(dz);
     if (lane < 16) red[c + lane] = sb;
+    bits = next;
   }
 }
 
@@ -367,6 +371,8 @@ __device__ __forceinline__ void out_epilogue(bool& ok, const OutLayer& o, uint32
   // and the row dot is added as two CTAs of half the columns add it: the same
   // order, the same bits.
   const bool whole = NT == N && (NT == 128 || NT == 256);
+  const bool valid = j < o.batch;
+  const float target = valid ? __ldg(o.y + j) : 0.0f, bias_out = __ldg(o.bL);  // (early: they are needed in a chain)
   if (ok) {
     float dot = 0.0f, first = 0.0f;  // (two names: an indexed pair would live in local memory)
     for (int c = cbeg; c < cbeg + cw; c += 16) {
@@ -403,12 +409,11 @@ __device__ __forceinline__ void out_epilogue(bool& ok, const OutLayer& o, uint32
         whole ? lo + (((E.rowq[512 + tid] + E.rowq[640 + tid]) + E.rowq[768 + tid]) + E.rowq[896 + tid]) : lo;
   }
   const float tot = totals.total(ok, E);
-  if (ok && tid < kM) E.yrow[tid] = tot + __ldg(o.bL);
+  if (ok && tid < kM) E.yrow[tid] = tot + bias_out;
   totals.settle(ok);
   if (ok) {
-    const bool valid = j < o.batch;
     const float yhat = E.yrow[r];
-    const float e = valid ? yhat - __ldg(o.y + j) : 0.0f;
+    const float e = valid ? yhat - target : 0.0f;
     const float dzL = valid ? 2.0f * e / (float)o.batch : 0.0f;
     const float rd = round_bf16(dzL);
     if (ns == 0 && cq == 0) {
@@ -662,8 +667,9 @@ __device__ __forceinline__ bool tr_tile(const TrArgs& args, int bid, uint8_t* sm
     fwd_cols<EMB>(tmem + lane_addr, E.s_bias, cbeg, cw, OwnRow{S1}, S2, NT, r, mask_out, J.rows_pad, drop, h1,
              ((uint64_t)j << 20) | (uint64_t)n0, args.drop_thr, args.drop_scale);
   } else if (ok && J.epi == TE_DX) {
-    dx_cols(tmem + lane_addr, cbeg, cw, OwnRow{J.out ? S1 : nullptr}, S2, NT, r, J.mask_in + (int64_t)(n0 >> 4) * J.rows_pad + j,
-            J.rows_pad, J.drop_h > 0 ? args.drop_scale : 1.0f, E.red + q * 256);
+    const uint16_t* mask = J.mask_in + (int64_t)(n0 >> 4) * J.rows_pad + j;
+    dx_cols(tmem + lane_addr, cbeg, cw, OwnRow{J.out ? S1 : nullptr}, S2, NT, r, mask, J.rows_pad,
+            mask[(int64_t)(cbeg >> 4) * J.rows_pad], J.drop_h > 0 ? args.drop_scale : 1.0f, E.red + q * 256);
     __syncthreads();
     for (int c = tid; c < NT; c += kT)
       J.colpart[(int64_t)mt * N + n0 + c] = col_total(E.red, c);
@@ -763,12 +769,13 @@ __global__ void __launch_bounds__(kT, 1) k_tr_gemm(const __grid_constant__ TrArg
 // (11K for the output layer's).  Before, each product was a launch of its own,
 // 5.5-8 us with its prologue, loads and tail.  A step (this, the gather, the
 // weight gradients and the optimiser; us, a launch per product -> now):
-//   128-256-256-256-1  batch 4096  49.8 -> 41.8     64-128-128-128-1  512  34.4 -> 25.9
-//   64-128-128-128-1   batch 4096, dropout  41.0 -> 32.8              8192  50.0 -> 32.8
-//   128-192-192-1      batch 8192  43.2 -> 34.0     128-256-256-1     8192  51.1 -> 34.5
-//   128-256-256-1      batch 4096  35.5 -> 31.2     16-64-1           256  16.2 -> 16.0
+//   128-256-256-256-1  batch 4096  49.8 -> 40.7     64-128-128-128-1  512  34.4 -> 25.4
+//   64-128-128-128-1   batch 4096, dropout  41.0 -> 32.3              8192  50.0 -> 32.2
+//   128-192-192-1      batch 8192  43.2 -> 33.3     128-256-256-1     8192  51.1 -> 33.8
+//   128-256-256-1      batch 4096  35.5 -> 30.6     16-64-1           256  16.2 -> 15.7
 // (of which the weight gradients' row copies, see copy_tile: 46.0 -> 41.8 for
-// the first, 37.2 -> 34.0 and 37.7 -> 34.5 for the third row).
+// the first, 37.2 -> 34.0 and 37.7 -> 34.5 for the third row; and the mask
+// words and targets requested before they are needed, about 1 us of each).
 constexpr int kMaxPhases = 2 * (LS_MAX_LAYERS - 1);
 constexpr int kMaxRing = 8;
 constexpr int kChainT = kT + 64;  // the epilogue's warps, the products' warp, the weights' warp
@@ -946,13 +953,15 @@ __global__ void __launch_bounds__(kChainT, 1) k_tr_chain(const __grid_constant__
         if (P.bias) E.s_bias[t] = __ldg(P.bias + n0 + t);
         if (P.epi == TE_FWD_OUT) E.s_w[t] = round_bf16(__ldg(a.wL + n0 + t));
       }
+      const int cw = NT / 4, cbeg = cq * cw, own0 = n0 / 64;
+      uint16_t* mask = P.mask + j + (int64_t)(n0 >> 4) * a.R;
+      const uint32_t bits = P.epi == TE_DX ? mask[(int64_t)(cbeg >> 4) * a.R] : 0u;
       if (tid == 0) bulk_commit_wait_read();  // the last product's stores have read S2
       __syncwarp();
       if (!mbar_wait(done, (uint32_t)p & 1u)) ok = false;
       ok = named_bar_and(1, kT, ok && !*gave_up);  // one decision for the whole CTA
       if (!ok) break;
       tc_fence_after();
-      const int cw = NT / 4, cbeg = cq * cw, own0 = n0 / 64;
       uint8_t* S1 = A + (size_t)((p + 1) & 1) * a.a_bytes + (size_t)own0 * kM * 128;
       uint64_t* sb = afull + ((p + 1) & 1) * kMaxChunks + own0;
       const bool send = CL > 1 && P.feeds;
@@ -962,7 +971,6 @@ __global__ void __launch_bounds__(kChainT, 1) k_tr_chain(const __grid_constant__
       // of the operand just read: the other rank writes none of them, and this
       // one not before its next epilogue
       uint8_t* S2 = A + (size_t)(p & 1) * a.a_bytes + (size_t)own0 * kM * 128;
-      uint16_t* mask = P.mask + j + (int64_t)(n0 >> 4) * a.R;
       if (P.epi == TE_FWD) {
         uint64_t h1 = 0;
         const bool drop = P.drop_h > 0;
@@ -973,7 +981,7 @@ __global__ void __launch_bounds__(kChainT, 1) k_tr_chain(const __grid_constant__
         fwd_cols<false>(taddr, E.s_bias, cbeg, cw, row, S2, NT, r, mask, a.R, drop, h1,
                         ((uint64_t)j << 20) | (uint64_t)n0, a.drop_thr, a.drop_scale);
       } else if (P.epi == TE_DX) {
-        dx_cols(taddr, cbeg, cw, row, S2, NT, r, mask, a.R, P.drop_h > 0 ? a.drop_scale : 1.0f, E.red + q * 256);
+        dx_cols(taddr, cbeg, cw, row, S2, NT, r, mask, a.R, bits, P.drop_h > 0 ? a.drop_scale : 1.0f, E.red + q * 256);
       } else {
         OutLayer o = a.out;
         o.colpart = P.colpart;
