@@ -35,6 +35,7 @@
 // instructions that each step runs once bound it.
 #include "blockhash.cuh"
 #include "common.cuh"
+#include "seq_steps.h"
 #include "sm100.cuh"
 
 namespace ls {
@@ -548,7 +549,7 @@ __global__ void __launch_bounds__(kSeqThreads, 1) k_route_seq(const __grid_const
   // The bids of request s: slot set s % 4, barrier s % 4 (its phase s / 4).
   // A set is written again four requests later, by CTAs that have this CTA's
   // bids of the three requests between, which it sends only after its own
-  // warps are done reading the set (named barriers 2 to 6 below).
+  // warps are done reading the set (the barriers of seq_steps.h).
   for (int e = tid; e < 256; e += kSeqThreads) cand[e] = ~0ull;  // slots of warps without a row keep this
   if (tid == 0) {
     *gave_up = 0;
@@ -603,21 +604,18 @@ __global__ void __launch_bounds__(kSeqThreads, 1) k_route_seq(const __grid_const
 #pragma unroll 1
     for (int s = 0; s <= a.n_req; ++s) {
       // Request s is looked up, request s - 3 inserted by this CTA's warps.
-      // (Barriers in turn, so that an arrival never meets an earlier round of
-      // its barrier: the next one on it comes after the bids of request s, or
-      // of s - 1 for the three of the inserting warps, sent after this point.)
+      // (Which barriers, and why no arrival meets an earlier use of its
+      // barrier: seq_steps.h.)
       __syncwarp();
-      if (s < a.n_req) {
-        named_bar_sync(2 + (s & 1), kSeqHalf + kSeqLook);
-        if (s >= 2) named_bar_sync(4 + (s - 2) % 3, kSeqHalf + kSeqIns);
-      }
+      if (s < a.n_req) named_bar_sync(seq::bar_looked_up(s), kSeqHalf + kSeqLook);
+      if (seq::waits_inserted(s, a.n_req)) named_bar_sync(seq::bar_inserted(s - 2), kSeqHalf + kSeqIns);
       if (s > 0) {
         if (lane == 0) seq_wait(&bar[(s - 1) & 3], (uint32_t)((s - 1) >> 2) & 1u, gave_up, a.err);
         __syncwarp();
         c1 = seq_select(cand + 64 * ((s - 1) & 3), slots);
         // the other warps may go on with this request's step
-        if (s + 1 < a.n_req) named_bar_arrive(7, kSeqHalf + kSeqLook);
-        named_bar_arrive(8 + (s & 1), kSeqHalf + kSeqIns);
+        if (seq::tells_look(s, a.n_req)) named_bar_arrive(seq::bar_bids_look(), kSeqHalf + kSeqLook);
+        named_bar_arrive(seq::bar_bids_insert(s), kSeqHalf + kSeqIns);
       }
       uint8_t* Xs = X0 + (s & 1) * x0_bytes;
       // 1. the last commit's queue, and this request's pair features given it
@@ -727,7 +725,7 @@ __global__ void __launch_bounds__(kSeqThreads, 1) k_route_seq(const __grid_const
       c2 = c1;
       if (s > 0) {  // the bids for request s - 1 are in
         __syncwarp();
-        named_bar_sync(7, kSeqHalf + kSeqLook);
+        named_bar_sync(seq::bar_bids_look(), kSeqHalf + kSeqLook);
         c1 = seq_select(cand + 64 * ((s - 1) & 3), slots);
       }
 #pragma unroll
@@ -768,7 +766,7 @@ __global__ void __launch_bounds__(kSeqThreads, 1) k_route_seq(const __grid_const
       }
       __syncwarp();
       named_bar_sync(10, kSeqLook);  // the masks are read
-      named_bar_arrive(2 + ((s + 1) & 1), kSeqHalf + kSeqLook);
+      named_bar_arrive(seq::bar_looked_up(s + 1), kSeqHalf + kSeqLook);
 #pragma unroll
       for (int q = 0; q < 5; ++q)
 #pragma unroll
@@ -792,7 +790,7 @@ __global__ void __launch_bounds__(kSeqThreads, 1) k_route_seq(const __grid_const
         int64_t b = (((int64_t)(it >> 5) * ranks + rank) << 5) + lane;
         uint64_t key = b < nb && k0 + b < a.bcap ? a.bkeys[k0 + b] : 0ull;
         __syncwarp();
-        named_bar_sync(8 + (s & 1), kSeqHalf + kSeqIns);  // the bids for request s - 1 are in
+        named_bar_sync(seq::bar_bids_insert(s), kSeqHalf + kSeqIns);  // the bids for request s - 1 are in
         const int c = seq_select(cand + 64 * ((s - 1) & 3), slots);
         int fresh = 0;
 #pragma unroll 1
@@ -805,10 +803,10 @@ __global__ void __launch_bounds__(kSeqThreads, 1) k_route_seq(const __grid_const
         if (lane == 0 && fresh && (int64_t)atomicAdd(a.counts + c, fresh) + fresh > a.max_keys)
           latch_error(a.err, LS_ERR_TABLE_FULL);
       }
-      if (s + 2 < a.n_req) {
+      if (seq::tells_inserted(s, a.n_req)) {
         __threadfence();  // the inserted keys before this CTA's next bids
         __syncwarp();
-        named_bar_arrive(4 + s % 3, kSeqHalf + kSeqIns);
+        named_bar_arrive(seq::bar_inserted(s), kSeqHalf + kSeqIns);
       }
     }
   }

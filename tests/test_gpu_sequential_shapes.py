@@ -34,6 +34,8 @@ CASES = [  # instances, state columns, extras, hidden, dtype, long prompts
     (9, 34, 24, (256, 256), "bf16", True), (17, 4, 3, (40,), "bf16", True), (33, 10, 0, (64, 64), "f32", True),
     (16, 66, 56, (512, 512), "bf16", False), (70, 10, 2, (64, 32), "bf16", True), (130, 4, 2, (48,), "f32", True),
     (300, 4, 2, (16, 16), "bf16", True), (5, 3, 1, (), "f32", False),
+    # a step that is shorter than its inserts: one instance, no hidden layer, hundreds of blocks
+    (1, 3, 1, (), "f32", True), (1, 3, 1, (), "bf16", True),
 ]
 
 
