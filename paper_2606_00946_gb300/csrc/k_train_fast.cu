@@ -25,6 +25,7 @@
 #include <cmath>
 
 #include "blockhash.cuh"
+#include "chain_tiles.h"
 #include "common.cuh"
 #include "sm100.cuh"
 
@@ -758,7 +759,8 @@ __global__ void __launch_bounds__(kT, 1) k_tr_gemm(const __grid_constant__ TrArg
 // into both CTAs' copies, the other's counted on its barriers.  Two copies in
 // turn need no cluster barrier: a rank writes the operand of product p + 1
 // once its own product p is done, so after the other has finished product
-// p - 1, which read that copy last.  Weights stream through a ring of K-blocks
+// p - 1, which read that copy last; the tile that the other may still be
+// storing from there keeps out of the way (chain_tiles.h).  Weights stream through a ring of K-blocks
 // that is filled ahead across products by a warp of its own; another issues
 // the products; sixteen run the epilogues.  Global memory gets only what the
 // weight gradients read, the transposed images.  Same tiles, products and
@@ -953,7 +955,7 @@ __global__ void __launch_bounds__(kChainT, 1) k_tr_chain(const __grid_constant__
         if (P.bias) E.s_bias[t] = __ldg(P.bias + n0 + t);
         if (P.epi == TE_FWD_OUT) E.s_w[t] = round_bf16(__ldg(a.wL + n0 + t));
       }
-      const int cw = NT / 4, cbeg = cq * cw, own0 = n0 / 64;
+      const int cw = NT / 4, cbeg = cq * cw, own0 = chain::first_block(rank, NT);
       uint16_t* mask = P.mask + j + (int64_t)(n0 >> 4) * a.R;
       const uint32_t bits = P.epi == TE_DX ? mask[(int64_t)(cbeg >> 4) * a.R] : 0u;
       if (tid == 0) bulk_commit_wait_read();  // the last product's stores have read S2
@@ -967,10 +969,12 @@ __global__ void __launch_bounds__(kChainT, 1) k_tr_chain(const __grid_constant__
       const bool send = CL > 1 && P.feeds;
       const ClusterRow row{P.feeds ? S1 : nullptr, send ? map_cluster(S1, (uint32_t)rank ^ 1u) : 0,
                            send ? map_cluster(sb, (uint32_t)rank ^ 1u) : 0};
-      // the transposed tile for its bulk stores takes this CTA's own columns
-      // of the operand just read: the other rank writes none of them, and this
-      // one not before its next epilogue
-      uint8_t* S2 = A + (size_t)(p & 1) * a.a_bytes + (size_t)own0 * kM * 128;
+      // the transposed tile for its bulk stores takes K-blocks of the operand
+      // just read that the other rank does not write for the next product (it
+      // may be at that epilogue already); this one writes there only in its
+      // own next epilogue, after the stores have read the tile
+      const int s2 = chain::stage_block(CL, rank, NT, p + 1 < a.n ? a.ph[p + 1].NT : NT);
+      uint8_t* S2 = A + (size_t)(p & 1) * a.a_bytes + (size_t)s2 * kM * 128;
       if (P.epi == TE_FWD) {
         uint64_t h1 = 0;
         const bool drop = P.drop_h > 0;

@@ -1,7 +1,7 @@
 """The training step's forward and input-gradient passes in one launch: the
 same bits as the persistent step, whose products run one after the other over
 the whole batch, for clusters of one and two CTAs a tile, layers of unlike
-widths, one layer to four, short last tiles, dropout and a bad slot."""
+widths (two to four of them), one layer to four, short last tiles, dropout and a bad slot."""
 import pytest
 import torch
 
@@ -22,6 +22,10 @@ CASES = [  # hidden, instance and request widths, batch, dropout
     ((256, 128), 34, 24, 257, 0.1), ((128, 256), 34, 24, 640, 0.1), ((64, 192), 34, 24, 384, 0.0),
     ((192, 192), 66, 56, 4096, 0.1), ((128, 128, 128), 34, 24, 4096, 0.1), ((128, 128), 34, 24, 10000, 0.0),
     ((256, 256, 256), 66, 56, 4096, 0.0), ((256, 256, 256, 256), 66, 56, 130, 0.1),
+    # clusters of two whose columns of one product are not those of the next, three and four products in a row
+    ((128, 256, 256), 34, 24, 8192, 0.0), ((256, 128, 128), 34, 24, 8192, 0.1), ((256, 256, 128), 34, 24, 4096, 0.0),
+    ((128, 128, 256), 34, 24, 4096, 0.1), ((256, 128, 256), 120, 120, 9000, 0.0),
+    ((128, 256, 128, 256), 34, 24, 8192, 0.1), ((256, 128, 128, 256), 10, 3, 4096, 0.0),
 ]
 
 
