@@ -157,7 +157,10 @@ __device__ __forceinline__ void seq_remote_store(uint32_t slot, uint32_t bar, ui
 }
 
 // Waits (bounded) for the bids of a request; once a wait of the CTA has given
-// up, none waits any more and the call runs to its end (error latched).
+// up, none waits any more and the call runs to its end (error latched).  From
+// then on the CTA sends no bids, so the others, each after its own wait, stop
+// too instead of joining bids of different requests; every CTA comes to the
+// cluster barrier at the kernel's end, and none leaves before it.
 __device__ __forceinline__ void seq_wait(uint64_t* bar, uint32_t parity, volatile int* gave_up, int* err) {
   if (mbar_try_wait(bar, parity)) return;
   const long long t0 = clock64();
@@ -599,7 +602,8 @@ __global__ void __launch_bounds__(kSeqThreads, 1) k_route_seq(const __grid_const
       slot_at = dsmem_addr(const_cast<const uint64_t*>(cand) + seen, (uint32_t)lane);
       bar_at = dsmem_addr(bar, (uint32_t)lane);
     }
-    int c1 = -1;  // where request s - 1 went
+    int c1 = -1;        // where request s - 1 went
+    bool sends = true;  // no wait of this CTA has given up
     seq_half_sync();  // X0 and the weights are complete
 #pragma unroll 1
     for (int s = 0; s <= a.n_req; ++s) {
@@ -610,8 +614,9 @@ __global__ void __launch_bounds__(kSeqThreads, 1) k_route_seq(const __grid_const
       if (s < a.n_req) named_bar_sync(seq::bar_looked_up(s), kSeqHalf + kSeqLook);
       if (seq::waits_inserted(s, a.n_req)) named_bar_sync(seq::bar_inserted(s - 2), kSeqHalf + kSeqIns);
       if (s > 0) {
-        if (lane == 0) seq_wait(&bar[(s - 1) & 3], (uint32_t)((s - 1) >> 2) & 1u, gave_up, a.err);
+        if (lane == 0 && sends) seq_wait(&bar[(s - 1) & 3], (uint32_t)((s - 1) >> 2) & 1u, gave_up, a.err);
         __syncwarp();
+        sends = !*gave_up;
         c1 = seq_select(cand + 64 * ((s - 1) & 3), slots);
         // the other warps may go on with this request's step
         if (seq::tells_look(s, a.n_req)) named_bar_arrive(seq::bar_bids_look(), kSeqHalf + kSeqLook);
@@ -672,7 +677,8 @@ __global__ void __launch_bounds__(kSeqThreads, 1) k_route_seq(const __grid_const
         bid = code < bid ? code : bid;
         if (lane == 0) sc[i] = z;
       }
-      if (warp < rows && lane < (int)ranks) seq_remote_store(slot_at + 512u * (s & 3), bar_at + 8u * (s & 3), bid);
+      if (warp < rows && lane < (int)ranks && sends)
+        seq_remote_store(slot_at + 512u * (s & 3), bar_at + 8u * (s & 3), bid);
       __syncwarp();
       if (lane == 0)
 #pragma unroll 1
@@ -810,6 +816,9 @@ __global__ void __launch_bounds__(kSeqThreads, 1) k_route_seq(const __grid_const
       }
     }
   }
+  __syncwarp();
+  cluster_sync();  // no CTA leaves while another may still store bids into it
+  if (*gave_up) cluster_drain();
 }
 
 }  // namespace

@@ -1015,6 +1015,7 @@ __global__ void __launch_bounds__(kChainT, 1) k_tr_chain(const __grid_constant__
   __syncwarp();
   __syncthreads();
   if (CL > 1) cluster_sync();  // no rank leaves while the other may still store to it
+  if (CL > 1 && *gave_up) cluster_drain();
   tc_fence_after();
   if (warp == 0) tmem_dealloc(tmem, a.tmem_cols);
 }

@@ -170,6 +170,15 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// For a CTA that gave up waiting for another one's asynchronous stores: after
+// the cluster barrier behind which none is issued, time for those under way to
+// land before it leaves (they take well under a microsecond; this is over 30).
+__device__ __forceinline__ void cluster_drain() {
+  const long long t0 = clock64();
+  while (clock64() - t0 < 65536) {
+  }
+}
+
 // fp32 at the same shared-memory offset in CTA `rank` of the cluster
 __device__ __forceinline__ float ld_dsmem_f32(const void* local, uint32_t rank) {
   uint32_t remote;
