@@ -7,6 +7,8 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
+
 #include "common.cuh"
 
 using namespace ls;
@@ -41,6 +43,22 @@ int cuda_fail(cudaError_t e, const char* where) {
 }  // namespace
 
 namespace ls {
+uint64_t cuda_context_id() {
+  typedef CUresult (*GetId)(CUcontext, unsigned long long*);
+  static const GetId get_id = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult found{};
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      return (GetId) nullptr;
+    }
+    return reinterpret_cast<GetId>(p);
+  }();
+  unsigned long long id = 0;
+  return get_id && get_id(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
 // Message for ls_last_error() from entry points defined in other files.
 void set_last_error(const char* msg) { g_err = msg; }
 }  // namespace ls
@@ -314,8 +332,6 @@ int ls_create(const ls_config* cfg, ls_ctx** out) {
     if (e == cudaSuccess) train_fast_bind(m, c.tf, c.tf.base, c.tf.parts);
     c.train_ctas = cfg->train_ctas > 0 && !c.tf.wide ? std::min(cfg->train_ctas, c.sms) : 0;
   }
-  A(c.use_tc ? prepare_score_tc(c.tc) : prepare_score_simt());
-  if (fast_train) A(prepare_train_fast(c.tf));
   if (e == cudaSuccess) {
     A(cudaEventCreateWithFlags(&c.ev_pub, cudaEventDisableTiming));
     A(cudaEventCreateWithFlags(&c.ev_route, cudaEventDisableTiming));

@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 #include <algorithm>
 #include <cstdint>
+#include <atomic>
 #include <mutex>
 #include <vector>
 
@@ -404,18 +405,36 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// Lets `kernel` take all the dynamic shared memory that its static part leaves
-// of a CTA's 227 KB.  Called for a context's kernels when it is created: the
-// attribute call costs the host about as much as a tenth of a launch, so it is
-// kept out of the calls (every context sets the same value, so none shrinks
-// what another relies on).
-template <typename... KArgs>
-cudaError_t allow_smem(void (*kernel)(KArgs...)) {
+// Number of the calling thread's CUDA context that no other one of the process
+// has or had (0: unknown).
+uint64_t cuda_context_id();
+
+// Lets kernel K take all the dynamic shared memory that its static part leaves
+// of a CTA's 227 KB, before a launch with more than 48 KB.  The limit belongs to
+// the CUDA context, not to a library context, so every call sets the same value
+// and none shrinks what another, in another thread, is about to launch with.
+// Done once per kernel and CUDA context and then known by the context's number:
+// the two runtime calls cost the host nearly 3 us, and a kernel that is not
+// launched is not loaded (loading all that a library context may launch when it
+// is created took the first of a process 0.93-0.97 ms where 0.31 was enough).
+template <auto* K>
+cudaError_t allow_smem() {
+  static std::atomic<uint64_t> done{0};
+  const uint64_t id = cuda_context_id();
+  if (id != 0 && done.load(std::memory_order_acquire) == id) return cudaSuccess;
   cudaFuncAttributes fa{};
-  const cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              227 * 1024 - (int)fa.sharedSizeBytes);
+  cudaError_t e = cudaFuncGetAttributes(&fa, K);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - (int)fa.sharedSizeBytes);
+  if (e == cudaSuccess) done.store(id, std::memory_order_release);
+  return e;
+}
+
+// launch_chained of a kernel that takes more than 48 KB of shared memory.
+template <auto* K, typename... Args>
+cudaError_t launch_smem(dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster, Args&&... args) {
+  const cudaError_t e = allow_smem<K>();
+  return e != cudaSuccess ? e : launch_chained(K, grid, block, smem, s, cluster, std::forward<Args>(args)...);
 }
 
 // ---------------------------------------------------------------------------
@@ -503,9 +522,6 @@ inline bool scorer_selects(const TcPlan& p, int n_req, int n_inst) {
   if (p.pair || p.wide) return false;
   return (n_inst <= 128 && 128 % n_inst == 0) || (int64_t)n_req * n_inst <= 128;
 }
-cudaError_t prepare_score_tc(const TcPlan& p);  // once per context, before its first launch
-cudaError_t prepare_score_simt();
-cudaError_t prepare_train_fast(const TrainFast& f);
 cudaError_t launch_score_tc(const MlpDesc& m, const TcPlan& p, const Published* pub, const int32_t* sel,
                             int n_req, int n_inst, const uint4* pairx, const uint8_t* ximg, int32_t* choice,
                             float* best,

@@ -321,8 +321,7 @@ cudaError_t launch_prefix_match(int n_req, const int32_t* tok, const int64_t* to
   if (n_req <= 0) return cudaSuccess;
   const size_t smem = (size_t)n_inst * 4 * sizeof(int32_t);
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_prefix_match, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    const cudaError_t e = allow_smem<k_prefix_match>();
     if (e != cudaSuccess) return e;
   }
   k_prefix_match<<<grid_for(n_req), kThreads, smem, s>>>(n_req, tok, tok_off, tables, mask, slots,

@@ -523,10 +523,8 @@ cudaError_t run_replay_admit(Ctx& c, float* d_out, float* n_out, cudaStream_t s)
     da.err = c.d_err;
     const int smem = 1024 + 3 * (H / 64) * kSlab + 8 * 64 * 4 + 128;
     e = traced(c, TR_REPLAY, 1, s, [&] {
-      cudaError_t a = cudaFuncSetAttribute(k_dist_rowmin, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (a != cudaSuccess) return a;
-      return launch_chained(k_dist_rowmin, dim3((tilesC + tilesK) * da.splits), dim3(kDistThreads), (size_t)smem, s, 1,
-                            da);
+      return launch_smem<k_dist_rowmin>(dim3((tilesC + tilesK) * da.splits), dim3(kDistThreads), (size_t)smem, s, 1,
+                                        da);
     });
     if (e != cudaSuccess) return e;
     e = traced(c, TR_REPLAY, 1, s, [&] {

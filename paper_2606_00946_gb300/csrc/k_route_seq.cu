@@ -840,6 +840,14 @@ size_t route_seq_smem(int n_inst, int d_inst, int wmax, int W) {
   return b <= 200 * 1024 ? b : 0;
 }
 
+namespace {
+template <int W>
+cudaError_t seq_kernel(bool bf16, void (*&k)(const SeqArgs)) {
+  k = bf16 ? k_route_seq<W, true> : k_route_seq<W, false>;
+  return bf16 ? allow_smem<k_route_seq<W, true>>() : allow_smem<k_route_seq<W, false>>();
+}
+}  // namespace
+
 cudaError_t launch_route_seq(int n_req, int n_inst, int d_inst, int d_req, int q_col, const int64_t* tok_off,
                              const uint64_t* bkeys, int64_t bcap, const float* req, float* inst, const float* mean,
                              const float* stdv, const Published* pub, const DevState* st, const MlpDesc& m,
@@ -896,14 +904,13 @@ cudaError_t launch_route_seq(int n_req, int n_inst, int d_inst, int d_req, int q
   a.wbytes = a.wsm ? (int64_t)wb : 0;
   const size_t smem = a.wsm ? with_w : seq_smem(a.rows, d_inst, a.xs, W, xe, a.hidden_out, 0).total;
   void (*k)(const SeqArgs) = nullptr;
+  cudaError_t e = cudaErrorInvalidValue;
   switch (W) {
-    case 1: k = m.bf16 ? k_route_seq<1, true> : k_route_seq<1, false>; break;
-    case 2: k = m.bf16 ? k_route_seq<2, true> : k_route_seq<2, false>; break;
-    case 4: k = m.bf16 ? k_route_seq<4, true> : k_route_seq<4, false>; break;
-    case 8: k = m.bf16 ? k_route_seq<8, true> : k_route_seq<8, false>; break;
-    default: return cudaErrorInvalidValue;
+    case 1: e = seq_kernel<1>(m.bf16, k); break;
+    case 2: e = seq_kernel<2>(m.bf16, k); break;
+    case 4: e = seq_kernel<4>(m.bf16, k); break;
+    case 8: e = seq_kernel<8>(m.bf16, k); break;
   }
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(ranks);

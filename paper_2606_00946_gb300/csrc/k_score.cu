@@ -478,13 +478,6 @@ SimtPlan plan_simt(const MlpDesc& m, int n_req, int n_inst, int sms) {
 
 bool simt_selects(const MlpDesc& m, int n_req, int n_inst, int sms) { return plan_simt(m, n_req, n_inst, sms).rq > 0; }
 
-cudaError_t prepare_score_simt() {
-  cudaError_t e = allow_smem(k_score_simt<4, true>);
-  if (e == cudaSuccess) e = allow_smem(k_score_simt<4, false>);
-  if (e == cudaSuccess) e = allow_smem(k_score_simt<8, true>);
-  return e == cudaSuccess ? allow_smem(k_score_simt<8, false>) : e;
-}
-
 cudaError_t launch_score_simt(const MlpDesc& mlp, const Published* pub, const int32_t* sel, int n_req, int n_inst,
                               const int64_t* tok_off, const int32_t* hits, const float* inst_state,
                               int d_inst, const float* req_feats, int d_req, const float* mean,
@@ -515,10 +508,12 @@ cudaError_t launch_score_simt(const MlpDesc& mlp, const Published* pub, const in
   a.scores = scores;
   a.choice = choice;
   a.best = best;
-  auto* k = p.tr <= 16 ? (p.staged ? k_score_simt<4, true> : k_score_simt<4, false>)
-                       : (p.staged ? k_score_simt<8, true> : k_score_simt<8, false>);
+  auto* launch = p.tr <= 16 ? (p.staged ? launch_smem<k_score_simt<4, true>, SimtArgs&>
+                                        : launch_smem<k_score_simt<4, false>, SimtArgs&>)
+                            : (p.staged ? launch_smem<k_score_simt<8, true>, SimtArgs&>
+                                        : launch_smem<k_score_simt<8, false>, SimtArgs&>);
   const int grid = (int)std::min<int64_t>(a.tiles, 2 * (int64_t)sms);
-  return launch_chained(k, dim3(grid), dim3(kSimtT), (size_t)p.smem, s, 1, a);
+  return launch(dim3(grid), dim3(kSimtT), (size_t)p.smem, s, 1, a);
 }
 
 cudaError_t launch_argmin(int n_req, int n_inst, const float* scores, int32_t* choice, float* best,

@@ -1900,29 +1900,18 @@ cudaError_t launch_feature_image(const int64_t* tok_off, const int32_t* hits, in
   const int nr_max = (kTileM + n_inst - 1) / n_inst + 1;  // requests a tile can touch
   const size_t smem = (size_t)nr_max * d_pad * sizeof(uint16_t);
   const int grid = (int)std::min<int64_t>(n_tiles, (int64_t)sms * 8);
+  if (smem > 48 * 1024) {
+    const cudaError_t e = allow_smem<k_feature_image>();
+    if (e != cudaSuccess) return e;
+  }
   return launch_chained(k_feature_image, dim3(grid), dim3(256), smem, s, 1, tok_off, hits, n_inst, xin, d_inst, d_req,
                         req, mean, stdv, d_pad, rows, n_tiles, nr_max, ximg);
-}
-
-cudaError_t prepare_score_tc(const TcPlan& p) {
-  if (p.pipe) {
-    const cudaError_t e = allow_smem(k_feature_image);
-    if (e != cudaSuccess) return e;
-    return allow_smem(k_score_tc_pipe);
-  }
-  if (p.pair) return allow_smem(p.n_tc == 3 ? k_score_pair<true> : k_score_pair<false>);
-  if (p.wide) {
-    const cudaError_t e = allow_smem(k_score_wide);
-    if (e != cudaSuccess) return e;
-  }
-  const cudaError_t e = allow_smem(k_score_tc<1>);
-  return e != cudaSuccess ? e : allow_smem(k_score_tc<2>);
 }
 
 int pair_max_clusters(const TcPlan& p) {
   if (!p.pair) return 0;
   auto kern = p.n_tc == 3 ? k_score_pair<true> : k_score_pair<false>;
-  if (allow_smem(kern) != cudaSuccess) return 0;
+  if ((p.n_tc == 3 ? allow_smem<k_score_pair<true>>() : allow_smem<k_score_pair<false>>()) != cudaSuccess) return 0;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1981,24 +1970,24 @@ cudaError_t launch_score_tc(const MlpDesc& m, const TcPlan& p, const Published* 
   a.n_tiles = (int)((rows + kTileM - 1) / kTileM);
   const int grid = std::min(a.n_tiles, sms);
   if (p.pipe) {
-    return launch_chained(k_score_tc_pipe, dim3(grid), dim3(kThreadsPipe), (size_t)p.pipe_smem, s, 1, a);
+    return launch_smem<k_score_tc_pipe>(dim3(grid), dim3(kThreadsPipe), (size_t)p.pipe_smem, s, 1, a);
   } else if (p.pair) {
     // the image is in the pair layout, which no other scorer reads
     if (!scores) return cudaErrorInvalidValue;
-    auto kern = p.n_tc == 3 ? k_score_pair<true> : k_score_pair<false>;
     const int tile_pairs = (a.n_tiles + 1) / 2;
     const int fit = p.pair_clusters > 0 ? p.pair_clusters : sms / 2;
     const int pairs = std::max(1, std::min(tile_pairs, fit));
-    return launch_chained(kern, dim3(2 * pairs), dim3(kThreadsPair), (size_t)p.pair_smem, s, 2, a);
+    auto* launch =
+        p.n_tc == 3 ? launch_smem<k_score_pair<true>, TcArgs&> : launch_smem<k_score_pair<false>, TcArgs&>;
+    return launch(dim3(2 * pairs), dim3(kThreadsPair), (size_t)p.pair_smem, s, 2, a);
   } else if (p.wide && scores) {
-    return launch_chained(k_score_wide, dim3(grid), dim3(kThreadsWide), (size_t)p.wide_smem, s, 1, a);
+    return launch_smem<k_score_wide>(dim3(grid), dim3(kThreadsWide), (size_t)p.wide_smem, s, 1, a);
   } else {
     if (!scores && !a.fuse_argmin) return cudaErrorInvalidValue;
     // two CTAs an SM where shared memory and the 512 TMEM columns hold both
     const bool two = p.smem <= 113 * 1024 && p.tmem_cols <= 256;
-    auto* kern = two ? k_score_tc<2> : k_score_tc<1>;
-    return launch_chained(kern, dim3(std::min(a.n_tiles, (two ? 2 : 1) * sms)), dim3(kThreadsTc), (size_t)p.smem, s, 1,
-                          a);
+    auto* launch = two ? launch_smem<k_score_tc<2>, TcArgs&> : launch_smem<k_score_tc<1>, TcArgs&>;
+    return launch(dim3(std::min(a.n_tiles, (two ? 2 : 1) * sms)), dim3(kThreadsTc), (size_t)p.smem, s, 1, a);
   }
 }
 

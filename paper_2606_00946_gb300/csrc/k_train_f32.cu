@@ -550,11 +550,8 @@ cudaError_t run_train_f32(Ctx& c, int B, const int32_t* idx, int opt, float lr, 
   a.err = c.d_err;
   const int ctas = std::min(a.tiles, c.sms);
   cudaError_t e = traced(c, TR_TRAIN_STEP, 1, s, [&] {
-    auto* k = a.tr == 4 ? k_trs_grad<4> : k_trs_grad<8>;
-    const int smem = (int)(floats * sizeof(float));
-    const cudaError_t r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (r != cudaSuccess) return r;
-    return launch_chained(k, dim3(ctas), dim3(kT), (size_t)smem, s, 1, a);
+    auto* launch = a.tr == 4 ? launch_smem<k_trs_grad<4>, TrsArgs&> : launch_smem<k_trs_grad<8>, TrsArgs&>;
+    return launch(dim3(ctas), dim3(kT), (size_t)floats * sizeof(float), s, 1, a);
   });
   if (e != cudaSuccess) return e;
   TrsOpt o{};

@@ -1541,16 +1541,17 @@ TrArgs tr_args(const Ctx& c, const TrJob& j0, const TrJob* j1, int* err) {
   return a;
 }
 
-cudaError_t launch_tr_args(const Ctx& c, const TrArgs& a, bool emb, cudaStream_t s) {
-  const TrJob& j0 = a.job[0];
-  const int n = a.n_cta;
-  const int smem = gemm_smem_bytes();
-  auto* k = emb ? (c.tf.wide ? k_tr_gemm<true, true> : k_tr_gemm<false, true>)
-                : (c.tf.wide ? k_tr_gemm<true, false> : k_tr_gemm<false, false>);
+template <bool RING, bool EMB>
+cudaError_t launch_tr_as(const TrArgs& a, cudaStream_t s) {
   // the column parts of a TE_FWD_OUT tile exchange row sums through
   // distributed shared memory: one cluster per tile
-  const int cl = j0.epi == TE_FWD_OUT ? j0.n_split : 1;
-  return launch_chained(k, dim3(n), dim3(kT), (size_t)smem, s, cl, a);
+  const int cl = a.job[0].epi == TE_FWD_OUT ? a.job[0].n_split : 1;
+  return launch_smem<k_tr_gemm<RING, EMB>>(dim3(a.n_cta), dim3(kT), (size_t)gemm_smem_bytes(), s, cl, a);
+}
+
+cudaError_t launch_tr_args(const Ctx& c, const TrArgs& a, bool emb, cudaStream_t s) {
+  if (emb) return c.tf.wide ? launch_tr_as<true, true>(a, s) : launch_tr_as<false, true>(a, s);
+  return c.tf.wide ? launch_tr_as<true, false>(a, s) : launch_tr_as<false, false>(a, s);
 }
 
 cudaError_t launch_tr_gemm(const Ctx& c, const TrJob& j0, const TrJob* j1, int* err, cudaStream_t s) {
@@ -1771,13 +1772,6 @@ GatherArgs gather_args(const Ctx& c, int B, const int32_t* idx) {
 }
 }  // namespace
 
-cudaError_t prepare_train_fast(const TrainFast& f) {
-  cudaError_t e = f.wide ? allow_smem(k_tr_gemm<true, false>) : allow_smem(k_tr_gemm<false, false>);
-  if (e == cudaSuccess) e = f.wide ? allow_smem(k_tr_gemm<true, true>) : allow_smem(k_tr_gemm<false, true>);
-  if (e == cudaSuccess) e = allow_smem(k_tr_chain);
-  return e == cudaSuccess ? allow_smem(k_tr_dw) : e;
-}
-
 cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr, float* loss_out, cudaStream_t s) {
   const MlpDesc& m = c.mlp;
   TrainFast& f = c.tf;
@@ -1946,13 +1940,13 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
     ca.drop_thr = t.drop_thr;
     ca.drop_scale = t.drop_scale;
     e = traced(c, TR_GEMM_TC_FWD, 1, s, [&] {
-      return launch_chained(k_tr_chain, dim3(T * cp.CL), dim3(kChainT), (size_t)cp.smem, s, cp.CL, ca);
+      return launch_smem<k_tr_chain>(dim3(T * cp.CL), dim3(kChainT), (size_t)cp.smem, s, cp.CL, ca);
     });
     if (e != cudaSuccess) return e;
     da.err = c.d_err;
     e = traced(c, TR_GEMM_TC_DW, 1, s, [&] {
       const int smem = 1024 + kDwStage + (2 * kMaxRing + 2) * 8;
-      return launch_chained(k_tr_dw, dim3(dw_ctas), dim3(kDwT), (size_t)smem, s, 1, da);
+      return launch_smem<k_tr_dw>(dim3(dw_ctas), dim3(kDwT), (size_t)smem, s, 1, da);
     });
     if (e != cudaSuccess) return e;
   }
@@ -1989,7 +1983,7 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
       cudaError_t e2 = cudaMemsetAsync(c.tr_bar, 0, 2 * sizeof(uint32_t), s);
       if (e2 != cudaSuccess) return e2;
       const int smem = gemm_smem_bytes();
-      e2 = cudaFuncSetAttribute(k_tr_step, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      e2 = allow_smem<k_tr_step>();
       if (e2 != cudaSuccess) return e2;
       cudaLaunchConfig_t cfg{};
       cfg.gridDim = dim3(c.train_ctas);

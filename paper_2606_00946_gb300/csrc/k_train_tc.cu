@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(kT) k_gemm_tc(const __grid_constant__ TcGemmAr
 
 template <int NTILE>
 cudaError_t run_tc(dim3 grid, int smem, const TcGemmArgs& g, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(k_gemm_tc<NTILE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const cudaError_t e = allow_smem<k_gemm_tc<NTILE>>();
   if (e != cudaSuccess) return e;
   k_gemm_tc<NTILE><<<grid, kT, smem, s>>>(g);
   return cudaGetLastError();
