@@ -293,8 +293,8 @@ int ls_create(const ls_config* cfg, ls_ctx** out) {
   // k_train_f32.cu, else the general step of k_train.cu)
   const bool fast_train = plan_train_fast(m, cfg->max_train_batch, c.tf);
   int64_t trs_floats = 0;
-  const bool trs = !fast_train && plan_train_f32(m, c.n_params, cfg->max_train_batch, c.sms, &trs_floats);
-  const bool general = !fast_train && !trs;
+  if (!fast_train) c.trs_batch = plan_train_f32(m, c.n_params, cfg->max_train_batch, c.sms, &trs_floats);
+  const bool general = !fast_train && cfg->max_train_batch > c.trs_batch;
   // replay admission embeds its records on the fast path's images, or through the general forward
   if (cfg->replay_capacity > 0 && c.rimg) {
     const int64_t tiles = (cfg->pending_capacity + 127) / 128 + (cfg->replay_capacity + 127) / 128;
@@ -313,7 +313,7 @@ int ls_create(const ls_config* cfg, ls_ctx** out) {
     c.gpart_floats = 64 * max_wl + 64 * (int64_t)m.max_width;  // dW partials, then column-sum partials
     A(dalloc(&c.gpart, c.gpart_floats));
   }
-  if (trs) A(dalloc(&c.trs_part, trs_floats));
+  if (c.trs_batch > 0) A(dalloc(&c.trs_part, trs_floats));
   A(dalloc(&c.loss_tmp, 1));
   A(dalloc(&c.d_err, 1));
   A(dalloc(&c.st, 1));
@@ -836,9 +836,9 @@ int ls_train_step(ls_ctx* h, int32_t batch, const int32_t* idx, int32_t opt, flo
   if (!c.have_params) return fail(LS_ERR_STATE, "parameters not set");
   if (!c.have_norm) return fail(LS_ERR_STATE, "normaliser not set");
   if (c.ring_enqueued < 1) return fail(LS_ERR_STATE, "sample ring is empty");
-  LS_CK(c.tf.on      ? run_train_fast(c, batch, idx, opt, lr, loss_out, S(stream))
-        : c.trs_part ? run_train_f32(c, batch, idx, opt, lr, loss_out, S(stream))
-                     : run_train_step(c, batch, idx, opt, lr, loss_out, S(stream)));
+  LS_CK(c.tf.on                ? run_train_fast(c, batch, idx, opt, lr, loss_out, S(stream))
+        : batch <= c.trs_batch ? run_train_f32(c, batch, idx, opt, lr, loss_out, S(stream))
+                               : run_train_step(c, batch, idx, opt, lr, loss_out, S(stream)));
   return LS_OK;
 }
 

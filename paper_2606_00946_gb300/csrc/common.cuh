@@ -278,7 +278,8 @@ struct Ctx {
   int64_t gpart_floats = 0;
   float* loss_tmp = nullptr;  // [1]
   TrainFast tf;               // tensor-core training buffers (when tf.on)
-  float* trs_part = nullptr;  // fp32 step (k_train_f32.cu): gradient partials per CTA (null: not used)
+  float* trs_part = nullptr;  // fp32 step in two launches (k_train_f32.cu): gradient partials per CTA
+  int trs_batch = 0;          // largest batch it takes (0: none; larger ones take the general path)
   int train_ctas = 0;         // > 0: persistent training step of that many CTAs
   uint32_t* tr_bar = nullptr; // [2]: its grid-barrier arrivals and abort flag
 
@@ -560,7 +561,7 @@ cudaError_t run_train_fast(Ctx& c, int batch, const int32_t* idx, int opt, float
                            cudaStream_t s);
 int64_t replay_embed_bytes(const MlpDesc& m, const TrainFast& f, int64_t rows);
 cudaError_t replay_embed_fast(Ctx& c, int64_t P, int64_t Rc, cudaStream_t s);
-bool plan_train_f32(const MlpDesc& m, int64_t n_params, int max_batch, int sms, int64_t* part_floats);
+int plan_train_f32(const MlpDesc& m, int64_t n_params, int max_batch, int sms, int64_t* part_floats);
 cudaError_t run_train_f32(Ctx& c, int batch, const int32_t* idx, int opt, float lr, float* loss_out,
                           cudaStream_t s);
 void set_last_error(const char* msg);  // sets the text ls_last_error() returns

@@ -23,6 +23,7 @@
 // two dZ buffers [out][rows].  When the weights do not all fit, a layer's are
 // staged in chunks of outputs as they are needed.
 #include <algorithm>
+#include <climits>
 
 #include "common.cuh"
 #include "sm100.cuh"
@@ -488,7 +489,7 @@ bool trs_plan(const MlpDesc& m, int B, int sms, int& tr, int& chunk, int64_t& fl
   for (int l = 0; l + 1 < m.n_layers; ++l) in_max = std::max<int64_t>(in_max, m.w[l]);
   const int64_t cap = kSmemMax / 4;
   tr = 4;
-  while (tr < 32 && (int64_t)(B + tr - 1) / tr > sms) tr *= 2;
+  while (tr < 32 && ((int64_t)B + tr - 1) / tr > sms) tr *= 2;
   for (; tr >= 4; tr /= 2) {
     const int64_t f = trs_floats(m, tr);
     for (int c : {0, 64, 32}) {
@@ -507,13 +508,37 @@ bool trs_plan(const MlpDesc& m, int B, int sms, int& tr, int& chunk, int64_t& fl
 
 // The fp32 step applies to fp32 predictors of at most kMaxParams parameters
 // whose activations fit in shared memory with a weight chunk.
-bool plan_train_f32(const MlpDesc& m, int64_t n_params, int max_batch, int sms, int64_t* part_floats) {
+//
+// Returns the largest batch it is taken for (0: none); the general path takes
+// larger ones.  A CTA shares a weight among the rows of one tile only, so every
+// further round of tiles costs as much as the first, in proportion to the
+// parameters; the general path pays some seven launches a layer once and its
+// products then fill the GPU.  The line: a 32-row tile per SM (fewer rows where
+// a tile has fewer), 16 rows where the layers average over 12K parameters, and
+// none for predictors that are small beside their layer count.  Device time of
+// a step as graph replays on 152 SMs, general path / this one, at or below the
+// line and above it:
+//   no line   64-64, d 16       166 / 103 us at 12,288 rows, 310 / 218 at 32,768
+//             80-80-80, d 64    338 / 284 at 16,384
+//   32 rows   128, d 64         70 / 46 at 4864       76 / 80 at 6144
+//             128-128-128, d 64 215 / 145 at 4864     240 / 307 at 6144
+//             160-160, d 64     175 / 138 at 4864     184 / 282 at 6144
+//   16 rows   192-96, d 128     135 / 62 at 2048      187 / 290 at 6144 (164 / 135 at 4096)
+//             512, d 64         64 / 61 at 2048       80 / 121 at 3072
+//             256-256, d 64     166 / 121 at 2048     198 / 250 at 3072
+//             1000, d 16 (tiles of 16)  56 / 43 at 1024  96 / 166 at 3072
+//   no hidden layer, 32 rows    25 / 25 at 4864       29 / 33 at 6144
+int plan_train_f32(const MlpDesc& m, int64_t n_params, int max_batch, int sms, int64_t* part_floats) {
   int tr, chunk;
   int64_t floats;
-  if (m.bf16 || n_params > kMaxParams || !trs_plan(m, 1, sms, tr, chunk, floats)) return false;
-  const int64_t ctas = std::min<int64_t>(sms, (max_batch + 3) / 4);
+  if (m.bf16 || n_params > kMaxParams || !trs_plan(m, 1, sms, tr, chunk, floats)) return 0;
+  trs_plan(m, INT_MAX, sms, tr, chunk, floats);  // tr: the rows of a tile of a large batch
+  const int64_t layers = m.n_layers;
+  const bool small = layers > 1 && n_params <= 1200 * layers * layers;
+  const int line = small ? INT_MAX : std::min(tr, n_params <= 12 * 1024 * layers ? 32 : 16) * sms;
+  const int64_t ctas = std::min<int64_t>(sms, (std::min(max_batch, line) + 3) / 4);
   *part_floats = ctas * (n_params + 2);
-  return true;
+  return line;
 }
 
 cudaError_t run_train_f32(Ctx& c, int B, const int32_t* idx, int opt, float lr, float* loss_out, cudaStream_t s) {
