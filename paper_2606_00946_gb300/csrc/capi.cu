@@ -520,7 +520,8 @@ int ls_snapshot_update(ls_ctx* h, int32_t n_inst, const float* inst_state, const
     }
     LS_CK(traced(c, TR_INDEX_INSERT, 1, S(stream), [&] {
       return launch_index_insert(keys, key_off, n_inst, n_keys, c.gkeys, c.gmask, c.gW, (uint64_t)(c.gslots - 1),
-                                 c.table_count, c.cfg.max_keys_per_instance, c.d_err, c.sms, S(stream));
+                                 c.table_count, c.cfg.max_keys_per_instance, mode == LS_REPLACE, c.d_err, c.sms,
+                                 S(stream));
     }));
   } else if (keys) {
     if (mode == LS_REPLACE) {

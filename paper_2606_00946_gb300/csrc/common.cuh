@@ -570,6 +570,6 @@ cudaError_t launch_prefix_index(int n_req, const int32_t* tok, const int64_t* to
                                 uint32_t* order, int sms, DevState* st, cudaStream_t s);
 cudaError_t launch_index_insert(const uint64_t* keys, const int64_t* key_off, int n_inst, int64_t n_keys,
                                 uint64_t* gkeys, uint64_t* gmask, int W, uint64_t gmask_slots, int32_t* counts,
-                                int64_t max_keys, int* err, int sms, cudaStream_t s);
+                                int64_t max_keys, bool cleared, int* err, int sms, cudaStream_t s);
 
 }  // namespace ls

@@ -491,14 +491,14 @@ __global__ void __launch_bounds__(1024) k_walk_order(int n_req, const int64_t* _
 // LS_ERR_TABLE_FULL, as does a probe sequence that finds no room).  With
 // W == 1 keys and masks share the interleaved entry array gkeys (gmask unused).
 //
-// A warp takes kInsU * 32 consecutive keys, so nearly every warp holds keys of
-// one instance: it finds that instance once and adds its distinct keys to the
-// instance's counter with one atomic.  (An atomic per key serialised on the
-// few counter addresses bounded the kernel: a rebuild of 32 instances of 16,384
-// keys with a 256-request route behind it took 384 us, 70 us with one per warp.)  A thread's kInsU first probes are in
-// flight together; what remains is two dependent L2 atomics per key.
-constexpr int kInsU = 4;
-
+// A warp takes U * 32 consecutive keys, so nearly every warp holds keys of one
+// instance: it finds that instance once and adds its distinct keys to the
+// instance's counter with one atomic.  (An atomic per key serialised on the few
+// counter addresses bounded the kernel: a rebuild of 32 instances of 16,384
+// keys with a 256-request route behind it took 384 us, 64 us with one per
+// warp.)  A thread's U first probes are in flight together; what remains is two
+// dependent L2 atomics per key.
+template <int U>
 __global__ void __launch_bounds__(256) k_index_insert(const uint64_t* __restrict__ keys,
                                                       const int64_t* __restrict__ key_off, int n_inst,
                                                       int64_t n_keys, uint64_t* gkeys, uint64_t* gmask, int W,
@@ -508,27 +508,27 @@ __global__ void __launch_bounds__(256) k_index_insert(const uint64_t* __restrict
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   unsigned long long* tab = reinterpret_cast<unsigned long long*>(gkeys);
   const int kstride = W == 1 ? 2 : 1;
-  for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; c * (32 * kInsU) < n_keys; c += warps) {
-    const int64_t base = c * (32 * kInsU);
+  for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; c * (32 * U) < n_keys; c += warps) {
+    const int64_t base = c * (32 * U);
     const int first = key_instance(key_off, n_inst, base);
     // (the last instance takes whatever follows its first key)
-    const bool one = first == n_inst - 1 || base + 32 * kInsU <= key_off[first + 1];
-    unsigned long long key[kInsU], prev[kInsU];
-    bool in[kInsU];
+    const bool one = first == n_inst - 1 || base + 32 * U <= key_off[first + 1];
+    unsigned long long key[U], prev[U];
+    bool in[U];
 #pragma unroll
-    for (int u = 0; u < kInsU; ++u) {
+    for (int u = 0; u < U; ++u) {
       const int64_t k = base + 32 * u + lane;
       in[u] = k < n_keys;
       key[u] = in[u] ? keys[k] : 0ull;
       if (key[u] == 0) key[u] = 1;
     }
 #pragma unroll
-    for (int u = 0; u < kInsU; ++u)
+    for (int u = 0; u < U; ++u)
       prev[u] = in[u] ? atomicCAS(tab + (key[u] & gmask_slots) * kstride, 0ull, key[u]) : 0ull;
-    bool fresh[kInsU];
-    int inst[kInsU];
+    bool fresh[U];
+    int inst[U];
 #pragma unroll
-    for (int u = 0; u < kInsU; ++u) {
+    for (int u = 0; u < U; ++u) {
       fresh[u] = false;
       inst[u] = one ? first : in[u] ? key_instance(key_off, n_inst, base + 32 * u + lane) : 0;
       if (!in[u]) continue;
@@ -551,12 +551,12 @@ __global__ void __launch_bounds__(256) k_index_insert(const uint64_t* __restrict
     if (one) {
       int n = 0;
 #pragma unroll
-      for (int u = 0; u < kInsU; ++u) n += __popc(__ballot_sync(kFull, fresh[u]));
+      for (int u = 0; u < U; ++u) n += __popc(__ballot_sync(kFull, fresh[u]));
       if (lane == 0 && n > 0 && (int64_t)atomicAdd(counts + first, n) + n > max_keys)
         latch_error(err, LS_ERR_TABLE_FULL);
     } else {
 #pragma unroll
-      for (int u = 0; u < kInsU; ++u)
+      for (int u = 0; u < U; ++u)
         if (fresh[u] && (int64_t)atomicAdd(counts + inst[u], 1) >= max_keys) latch_error(err, LS_ERR_TABLE_FULL);
     }
   }
@@ -619,11 +619,19 @@ cudaError_t launch_prefix_index(int n_req, const int32_t* tok, const int64_t* to
 
 cudaError_t launch_index_insert(const uint64_t* keys, const int64_t* key_off, int n_inst, int64_t n_keys,
                                 uint64_t* gkeys, uint64_t* gmask, int W, uint64_t gmask_slots, int32_t* counts,
-                                int64_t max_keys, int* err, int sms, cudaStream_t s) {
+                                int64_t max_keys, bool cleared, int* err, int sms, cudaStream_t s) {
   if (n_keys <= 0 || n_inst <= 0) return cudaSuccess;
-  const int64_t blocks = std::min<int64_t>((n_keys + 256 * kInsU - 1) / (256 * kInsU), (int64_t)sms * 32);
-  k_index_insert<<<(int)blocks, 256, 0, s>>>(keys, key_off, n_inst, n_keys, gkeys, gmask, W, gmask_slots, counts,
-                                             max_keys, err);
+  // Four keys a thread once a cleared table takes more keys than the GPU has
+  // threads (whole calls: 1,048,576 keys of 64 instances 39.7 us, 45.4 with one
+  // a thread; 2,000,000 of one 105, 136); one while threads are idle (100,000
+  // keys of one instance 22.9 us, 38.2 with four) and into a filled table, where
+  // the probes find their keys and the second atomic is the longer wait
+  // (2,000,000 keys already held 54 us, 85 with four).
+  const bool four = cleared && n_keys > (int64_t)sms * 2048;
+  const int64_t per = 256 * (four ? 4 : 1);
+  const int64_t blocks = std::min<int64_t>((n_keys + per - 1) / per, (int64_t)sms * 32);
+  auto* k = four ? k_index_insert<4> : k_index_insert<1>;
+  k<<<(int)blocks, 256, 0, s>>>(keys, key_off, n_inst, n_keys, gkeys, gmask, W, gmask_slots, counts, max_keys, err);
   return cudaGetLastError();
 }
 

@@ -60,3 +60,35 @@ def test_membership_and_distinct_counts(counts, spare):
         again = r.route(toks.reshape(-1), off, torch.zeros(n_req, 0, device="cuda"), n_inst)
         assert r.sync() == L.LS_OK
         assert np.array_equal(again["hits"].cpu().numpy(), want)
+
+
+# more keys than a GPU of 152 SMs has threads: four a thread into a cleared
+# table, one a thread into a filled one
+@pytest.mark.parametrize("counts", [[200_000, 0, 150_001], [330_000], [4000] * 70 + [40_000]])
+@pytest.mark.parametrize("spare", [0, -1])
+def test_many_keys(counts, spare):
+    n_inst, n_req = len(counts), 700
+    g = np.random.default_rng(sum(counts))
+    toks = torch.from_numpy(g.integers(0, 32000, size=(n_req, 16)).astype(np.int32)).cuda()
+    off = torch.arange(n_req + 1, dtype=torch.int64, device="cuda") * 16
+    r = router(n_inst, max(counts) + spare, n_req)
+    keys, _ = r.hash_blocks(toks.reshape(-1), off)
+    # each instance: some of the prompts' keys, the rest distinct others, in any order
+    held = [np.sort(g.choice(n_req, size=min(c, 300), replace=False)) for c in counts]
+    flat = []
+    for h, c in zip(held, counts):
+        fill = torch.from_numpy(g.integers(1 << 20, 1 << 62, size=c - len(h)) | 1).cuda()
+        k = torch.cat([keys[torch.from_numpy(h).cuda()], fill])
+        assert len(torch.unique(k)) == c
+        flat.append(k[torch.from_numpy(g.permutation(c)).cuda()])
+    koff = torch.tensor(np.concatenate([[0], np.cumsum(counts)]), dtype=torch.int64, device="cuda")
+    flat, state = torch.cat(flat), torch.zeros(n_inst, 10, device="cuda")
+    want = np.zeros((n_req, n_inst), np.int32)
+    for i, h in enumerate(held):
+        want[h, i] = 1
+    for mode in (L.LS_REPLACE, L.LS_INSERT):  # (the insert changes nothing)
+        r.snapshot(n_inst, state, flat, koff, mode=mode)
+        out = r.route(toks.reshape(-1), off, torch.zeros(n_req, 0, device="cuda"), n_inst)
+        assert r.sync() == (L.LS_OK if spare == 0 or mode == L.LS_INSERT else L.LS_ERR_TABLE_FULL)
+        assert np.array_equal(out["hits"].cpu().numpy(), want)
+    r.close()
