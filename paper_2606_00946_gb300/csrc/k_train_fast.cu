@@ -1807,6 +1807,17 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
     e = traced(c, TR_GATHER, 1, s, [&] {
       const int64_t total = (int64_t)R * (f.in_pad[0] / 8);
       const int grid = (int)std::min<int64_t>((total + 255) / 256, (int64_t)c.sms * 8);
+      // Long rows that are not whole 16-byte vectors are read word by word and
+      // live on L1, which an SM that still runs the step before has set to
+      // shared memory: then the gather waits for that step before it starts.
+      // (Steps issued one by one, 246-256-1: 8192 rows 42 us chained, 35 so;
+      // 32,768 rows 128, 102; 129-256-1 at 16,384 57, 50.  The chained launch is
+      // the faster one for short rows, 29-128-1 at 2048 rows 19 us against 21,
+      // and small batches.)
+      if ((m.w[0] & 3) != 0 && m.w[0] > 64 && R >= 2048) {
+        k_tr_gather<<<grid, 256, 0, s>>>(gather_args(c, B, idx));
+        return cudaGetLastError();
+      }
       return launch_chained(k_tr_gather, dim3(grid), dim3(256), 0, s, 1, gather_args(c, B, idx));
     });
     if (e != cudaSuccess) return e;
