@@ -275,12 +275,13 @@ int ls_create(const ls_config* cfg, ls_ctx** out) {
   A(dalloc(&c.ring_y, ring_rows));
   if (cfg->replay_capacity > 0) {
     const int64_t er = cfg->pending_capacity + cfg->replay_capacity;
-    A(dalloc(&c.remb, er * m.w[m.n_layers - 1]));
     A(dalloc(&c.rnorm, er));
     A(dalloc(&c.rpart, er * kRowMinParts));
     const int H = m.w[m.n_layers - 1];
     if (m.bf16 && H % 64 == 0 && H <= 256)  // tensor-core distances from a bf16 image
       A(dalloc(&c.rimg, ((cfg->pending_capacity + 127) / 128 + (cfg->replay_capacity + 127) / 128) * 128 * H * 2));
+    else
+      A(dalloc(&c.remb, er * H));
     A(dalloc(&c.rd, cfg->pending_capacity));
     A(dalloc(&c.rn, cfg->replay_capacity));
     A(dalloc(&c.rinv, er));

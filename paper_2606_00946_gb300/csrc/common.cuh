@@ -229,7 +229,7 @@ struct Ctx {
   float* ring_y = nullptr;
   int64_t replay_base = 0;        // C + P
   // replay admission scratch
-  float* remb = nullptr;          // embeddings [P + Rc, H] fp32 (candidates, then kept)
+  float* remb = nullptr;          // embeddings [P + Rc, H] fp32 (candidates, then kept), without an image (rimg)
   float* rnorm = nullptr;         // |bf16(g)|^2 [P + Rc] (+inf for rows not in use)
   float* rpart = nullptr;         // row-min partials [max(P, Rc), kRowMinParts]
   float* rd = nullptr;            // d per candidate [P]

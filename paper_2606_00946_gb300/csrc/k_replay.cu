@@ -96,11 +96,11 @@ __global__ void k_replay_gather(int B, int64_t row0, int d, ReplayGeom g, const 
   }
 }
 
-// One warp per compact row: g = (yhat - y) a_last (fp32) and |bf16(g)|^2
-// (summed in a fixed shuffle order) at its embedding row; rows the round does
-// not use keep the +inf norm k_replay_prep gave them (never nearest).  With an
-// image (bf16 distances on tensor cores) the bf16 row also goes to its
-// 128-row tile: candidate tiles first, then kept tiles.
+// One warp per compact row: g = (yhat - y) a_last and |bf16(g)|^2 (summed in a
+// fixed shuffle order); rows the round does not use keep the +inf norm
+// k_replay_prep gave them (never nearest).  g goes to its embedding row in fp32
+// or, with an image (bf16 distances on tensor cores), in bf16 to its 128-row
+// tile: candidate tiles first, then kept tiles.
 __global__ void k_replay_embed(int B, int64_t row0, int H, ReplayGeom g, const int64_t* __restrict__ counts,
                                const float* __restrict__ a_last, const float* __restrict__ yhat,
                                const float* __restrict__ y, float* __restrict__ emb, float* __restrict__ norm,
@@ -123,10 +123,10 @@ __global__ void k_replay_embed(int B, int64_t row0, int H, ReplayGeom g, const i
     }
     for (int k = lane; k < H; k += 32) {
       const float v = res * a_last[j * H + k];
-      emb[r * H + k] = v;
       const float b = round_bf16(v);
       s = fmaf(b, b, s);
       if (trow) *reinterpret_cast<__nv_bfloat16*>(trow + sm100::sw128_offset(rr, k, 128)) = __float2bfloat16_rn(v);
+      else emb[r * H + k] = v;
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
@@ -534,7 +534,7 @@ cudaError_t run_replay_admit(Ctx& c, float* d_out, float* n_out, cudaStream_t s)
     if (e != cudaSuccess) return e;
   }
   const float* Ec = c.remb;
-  const float* Ek = c.remb + g.P * H;
+  const float* Ek = Ec ? Ec + g.P * H : nullptr;
   const float* nc = c.rnorm;
   const float* nkp = c.rnorm + g.P;
   const int64_t kNoSelf = -(int64_t(1) << 62);
