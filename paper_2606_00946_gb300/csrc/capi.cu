@@ -601,9 +601,10 @@ int route_impl(ls_ctx* h, int32_t n_req, const int32_t* tok, const int64_t* tok_
                                                   : simt_selects(c.mlp, n_req, c.n_inst, c.sms));
   float* scores = scores_opt ? scores_opt : (fused_select ? nullptr : c.scores);
   if (c.use_index) {
-    LS_CK(traced(c, TR_PREFIX_INDEX, 1, s, [&] {
+    int launches = 1;
+    LS_CK(traced(c, TR_PREFIX_INDEX, launches, s, [&] {
       return launch_prefix_index(n_req, tok, tok_off, c.gkeys, c.gmask, c.gW, (uint64_t)(c.gslots - 1), c.n_inst,
-                                 hits, c.order, c.sms, c.st, s);
+                                 hits, c.order, c.sms, c.st, &launches, s);
     }));
   } else if (c.cfg.prefix_mode == LS_PREFIX_FUSED) {
     LS_CK(traced(c, TR_PREFIX, 1, s, [&] {

@@ -294,9 +294,10 @@ inline bool capturing(cudaStream_t s) {
   return cudaStreamIsCapturing(s, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
 }
 
-// Launch bracketed by trace events (skipped while the stream is being captured).
+// Launches bracketed by trace events (skipped while the stream is being
+// captured); f may change n_launch, their number, which is read after it.
 template <class F>
-cudaError_t traced(Ctx& c, int id, int n_launch, cudaStream_t s, F&& f) {
+cudaError_t traced(Ctx& c, int id, const int& n_launch, cudaStream_t s, F&& f) {
   const int t = c.tracer.on && !capturing(s) ? c.tracer.begin(s) : -1;
   const cudaError_t e = f();
   c.tracer.end(t, id, n_launch, s);
@@ -567,7 +568,7 @@ cudaError_t run_train_f32(Ctx& c, int batch, const int32_t* idx, int opt, float 
 void set_last_error(const char* msg);  // sets the text ls_last_error() returns
 cudaError_t launch_prefix_index(int n_req, const int32_t* tok, const int64_t* tok_off, const uint64_t* gkeys,
                                 const uint64_t* gmask, int W, uint64_t gmask_slots, int n_inst, int32_t* hits,
-                                uint32_t* order, int sms, DevState* st, cudaStream_t s);
+                                uint32_t* order, int sms, DevState* st, int* launches, cudaStream_t s);
 cudaError_t launch_index_insert(const uint64_t* keys, const int64_t* key_off, int n_inst, int64_t n_keys,
                                 uint64_t* gkeys, uint64_t* gmask, int W, uint64_t gmask_slots, int32_t* counts,
                                 int64_t max_keys, bool cleared, int* err, int sms, cudaStream_t s);

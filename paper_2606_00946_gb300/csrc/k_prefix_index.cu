@@ -568,7 +568,7 @@ int index_words(int max_instances) { return max_instances <= 64 ? 1 : max_instan
 
 cudaError_t launch_prefix_index(int n_req, const int32_t* tok, const int64_t* tok_off, const uint64_t* gkeys,
                                 const uint64_t* gmask, int W, uint64_t gmask_slots, int n_inst, int32_t* hits,
-                                uint32_t* order, int sms, DevState* st, cudaStream_t s) {
+                                uint32_t* order, int sms, DevState* st, int* launches, cudaStream_t s) {
   if (n_req <= 0) return cudaSuccess;
   void (*k)(int, const int32_t*, const int64_t*, const uint64_t*, const uint64_t*, uint64_t, int, int32_t*,
             DevState*, const uint32_t*) = nullptr;
@@ -609,6 +609,7 @@ cudaError_t launch_prefix_index(int n_req, const int32_t* tok, const int64_t* to
   // more requests than warps at once: the long ones first (8192 prompts of 8k
   // to 32k tokens over 64 instances: a route took 334 us in order, 318 so)
   const bool sorted = order && grid < want;
+  *launches = sorted ? 2 : 1;
   if (sorted) {
     const cudaError_t e = launch_chained(k_walk_order, dim3(1), dim3(1024), 0, s, 1, n_req, tok_off, order);
     if (e != cudaSuccess) return e;

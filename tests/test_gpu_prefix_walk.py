@@ -64,3 +64,21 @@ def test_hits_equal_the_two_phase_kernels(n_req, n_inst, max_len, shift):
     assert int(hits[0].max()) > 0
     for r in routers:
         r.close()
+
+
+def test_the_trace_counts_the_sort():
+    """A traced route's launches: the walk alone, or the sort by length before it."""
+    for n_req, want in ((64, 1), (1300, 1), (6000, 2)):
+        r = H.Router([16, 64, 1], 10, 0, "bf16", max_instances=4, max_requests=n_req, max_keys_per_instance=64,
+                     max_batch_tokens=16 * n_req, ring_capacity=16, max_train_batch=64)
+        r.set_normalizer(torch.zeros(16, device="cuda"), torch.ones(16, device="cuda"))
+        r.set_params(torch.zeros(r.n_params, device="cuda"))
+        r.snapshot(4, torch.zeros(4, 10, device="cuda"))
+        r.publish()
+        tok = torch.zeros(16 * n_req, dtype=torch.int32, device="cuda")
+        off = torch.arange(n_req + 1, dtype=torch.int64, device="cuda") * 16
+        assert L.ls_trace_enable(r.h, True) == L.LS_OK
+        r.route(tok, off, torch.zeros(n_req, 0, device="cuda"), 4)
+        rc, entries = L.ls_trace_read(r.h)
+        assert rc == L.LS_OK and entries["prefix_index"][0] == want, (n_req, entries)
+        r.close()
