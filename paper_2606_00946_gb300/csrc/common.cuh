@@ -322,6 +322,21 @@ __device__ __forceinline__ void route_snapshot(DevState* st) {
     st->route_b = *reinterpret_cast<volatile int32_t*>(&st->cur);
 }
 
+// sum_{s < n} src[s * stride], added in order, sixteen loads in flight.
+__device__ __forceinline__ float ordered_sum(const float* __restrict__ src, int n, int64_t stride) {
+  float g = 0.0f;
+  int s = 0;
+  for (; s + 16 <= n; s += 16) {
+    float v[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) v[u] = __ldg(src + (int64_t)(s + u) * stride);
+#pragma unroll
+    for (int u = 0; u < 16; ++u) g += v[u];
+  }
+  for (; s < n; ++s) g += __ldg(src + (int64_t)s * stride);
+  return g;
+}
+
 // True in exactly one block of the grid: the last to arrive at `done`, after
 // every block has passed this point (so every block's earlier reads of the
 // state it will update are done).  The counter is reset for the next launch.

@@ -588,7 +588,7 @@ cudaError_t launch_prefix_index(int n_req, const int32_t* tok, const int64_t* to
       case 1: c = wide ? k_prefix_index_coop<1, 8> : k_prefix_index_coop<1, 4>; break;
       case 2: c = wide ? k_prefix_index_coop<2, 8> : k_prefix_index_coop<2, 4>; break;
       case 4: c = wide ? k_prefix_index_coop<4, 8> : k_prefix_index_coop<4, 4>; break;
-      default: c = wide ? k_prefix_index_coop<8, 8> : k_prefix_index_coop<8, 4>; break;
+      default: c = k_prefix_index_coop<8, 8>; break;  // (at most a request per SM)
     }
     return launch_chained(c, dim3(n_req), dim3(wide ? 256 : 128), 0, s, 1, tok, tok_off, gkeys, gmask, gmask_slots,
                           n_inst, hits, st);

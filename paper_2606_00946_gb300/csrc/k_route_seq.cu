@@ -140,14 +140,6 @@ __device__ __forceinline__ uint64_t seq_code(float v, int i) {
   return ((uint64_t)c << 32) | (uint32_t)i;
 }
 
-// The address, in CTA `rank` of the cluster, of what lies at this shared-memory
-// address here.
-__device__ __forceinline__ uint32_t dsmem_addr(const void* local, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(local)), "r"(rank));
-  return r;
-}
-
 // v into the 64-bit word at `slot`, its eight bytes counted on the barrier at
 // `bar` (addresses in the same CTA of the cluster).
 __device__ __forceinline__ void seq_remote_store(uint32_t slot, uint32_t bar, uint64_t v) {
@@ -599,8 +591,8 @@ __global__ void __launch_bounds__(kSeqThreads, 1) k_route_seq(const __grid_const
     const int seen = (int)rank * min(R, kSeqWarps) + warp;
     uint32_t slot_at = 0, bar_at = 0;
     if (lane < (int)ranks) {
-      slot_at = dsmem_addr(const_cast<const uint64_t*>(cand) + seen, (uint32_t)lane);
-      bar_at = dsmem_addr(bar, (uint32_t)lane);
+      slot_at = map_cluster(const_cast<const uint64_t*>(cand) + seen, (uint32_t)lane);
+      bar_at = map_cluster(bar, (uint32_t)lane);
     }
     int c1 = -1;        // where request s - 1 went
     bool sends = true;  // no wait of this CTA has given up

@@ -403,21 +403,6 @@ struct TrsOpt {
   DevState* st;
 };
 
-// sum of the CTAs' partials of one value, in order, sixteen loads in flight
-__device__ __forceinline__ float trs_sum(const float* __restrict__ src, int n, int64_t stride) {
-  float g = 0.0f;
-  int s = 0;
-  for (; s + 16 <= n; s += 16) {
-    float v[16];
-#pragma unroll
-    for (int u = 0; u < 16; ++u) v[u] = __ldg(src + (int64_t)(s + u) * stride);
-#pragma unroll
-    for (int u = 0; u < 16; ++u) g += v[u];
-  }
-  for (; s < n; ++s) g += __ldg(src + (int64_t)s * stride);
-  return g;
-}
-
 __global__ void __launch_bounds__(128) k_trs_opt(const __grid_constant__ TrsOpt a) {
   pdl_wait();
   pdl_trigger();
@@ -433,7 +418,7 @@ __global__ void __launch_bounds__(128) k_trs_opt(const __grid_constant__ TrsOpt 
       vo = a.vo[e];
     }
     const float p = a.p[e];
-    const float g = trs_sum(a.part + e, a.parts, a.ld);
+    const float g = ordered_sum(a.part + e, a.parts, a.ld);
     if (!aborted) {
       if (a.adam) {
         const float me = 0.9f * mo + 0.1f * g;

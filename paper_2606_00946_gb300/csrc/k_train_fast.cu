@@ -1252,21 +1252,6 @@ __global__ void k_tr_gather(const __grid_constant__ GatherArgs g) {
                   blockIdx.x == 0 && threadIdx.x == 0);
 }
 
-// sum_{s < n} src[s * stride], added in order, sixteen loads in flight.
-__device__ __forceinline__ float ordered_sum(const float* __restrict__ src, int n, int64_t stride) {
-  float g = 0.0f;
-  int s = 0;
-  for (; s + 16 <= n; s += 16) {
-    float v[16];
-#pragma unroll
-    for (int u = 0; u < 16; ++u) v[u] = __ldg(src + (int64_t)(s + u) * stride);
-#pragma unroll
-    for (int u = 0; u < 16; ++u) g += v[u];
-  }
-  for (; s < n; ++s) g += __ldg(src + (int64_t)s * stride);
-  return g;
-}
-
 struct OptLayer {
   const float* partW;  // [S][out][ld] split partials of dW (hidden) or [T][in] tile partials (output)
   int S;
@@ -1296,9 +1281,6 @@ struct OptArgs {
   int blk0[LS_MAX_LAYERS + 1];
 };
 
-// Gradient of every parameter as an ordered sum of its partials, the
-// optimiser update of the fp32 master, and the bf16 images of the updated
-// hidden-layer weights, for parameters [first, n) with stride `stride`.
 // Gradient (ordered sum of its partials), optimiser update and bf16 image
 // writes of parameter e of layer l.  A step whose gather found no record or a
 // bad slot (`aborted`) changes nothing: the images already hold the unchanged
@@ -1354,7 +1336,8 @@ __device__ __forceinline__ void tr_opt_one(const OptArgs& a, int l, int64_t e, b
   }
 }
 
-// Every parameter in [first, n) with stride `stride` (the persistent step).
+// The gradient, the update of the fp32 master and the images of every parameter
+// in [first, n) with stride `stride` (the persistent step).
 __device__ __forceinline__ void tr_opt_items(const OptArgs& a, int64_t first, int64_t stride) {
   const MlpDesc& m = a.m;
   const int nl = m.n_layers;
