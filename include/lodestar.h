@@ -117,11 +117,14 @@ typedef struct {
     float dropout;
     uint64_t dropout_seed;
     /* Launch shape of a tensor-core training step (bf16, hidden widths <=
-     * 256): <= 0 uses one launch per phase (gather, each product, optimiser;
-     * the default and the faster one measured), > 0 runs the whole step as
-     * one persistent launch of that many CTAs (at most the SM count) that
-     * meet at a grid barrier between phases.  Results are the same bits
-     * either way. */
+     * 256): <= 0 uses four launches (gather, forward pass with the input
+     * gradients, weight gradients, optimiser), or a launch per product where
+     * the layers' widths do not split alike; the default and the faster one
+     * measured.  > 0 runs the whole step as one persistent launch of that
+     * many CTAs (at most the SM count) that meet at a grid barrier between
+     * phases.  Results are the same bits either way.  Without effect when a
+     * hidden layer is wider than 256 (384 and 512 run a launch per product;
+     * other widths and fp32 predictors do not train on tensor-core images). */
     int32_t train_ctas;
 } ls_config;
 

@@ -15,9 +15,20 @@
 //   last l     ... plus the width-1 output layer: yhat, loss, dz_L = 2 (yhat - y) / B,
 //              dW_L, db_L partials, dz_l = bf16(dz_L) bf16(w_L) [Z > 0] -> img(dz_l), img(dz_l^T)
 //   backward   dW_l = bf16(dz_l)^T A_l   (split over the batch, fp32 partials)
-//              dz_{l-1} = (bf16(dz_l) W_l) [Z_{l-1} > 0] -> images   (same launch)
+//              dz_{l-1} = (bf16(dz_l) W_l) [Z_{l-1} > 0] -> images
 //   optimiser  gradient = ordered sum of the partials; SGD / Adam on the fp32
 //              master; rewrites img(W_l), img(W_l^T) for the next step.
+// How these are launched depends on the shape (run_train_fast):
+//   hidden layers up to 256   gather; k_tr_chain: every forward layer, the output
+//                             layer and the input gradients, a 128-row tile's
+//                             activations kept in shared memory; k_tr_dw: the
+//                             weight gradients of every layer; optimiser
+//   what plan_chain refuses,  gather; k_tr_gemm per product, a weight gradient
+//   layers of 384 or 512      beside each input gradient; optimiser
+//   train_ctas > 0            one persistent launch, k_tr_step, the same products
+//                             as its phases
+// Replay admission runs the forward layers alone (k_emb_gather, k_tr_gemm,
+// k_emb_rows).
 // Bias gradients are column sums of the unrounded dz, formed per 128-row tile
 // in the epilogues.  The rounding points are those of the reference path
 // (k_train.cu): bf16 operands of every product, fp32 sums, biases and state.
