@@ -232,8 +232,10 @@ __device__ __forceinline__ void trs_dw(const float* dz, const float* x, float* p
   }
 }
 
+// (one CTA an SM is launched, so a thread may have 255 registers: held to 128
+// for a second one, the kernel spilled)
 template <int RV>
-__global__ void __launch_bounds__(kT) k_trs_grad(const __grid_constant__ TrsArgs a) {
+__global__ void __launch_bounds__(kT, 1) k_trs_grad(const __grid_constant__ TrsArgs a) {
   extern __shared__ __align__(16) float sm[];
   __shared__ float s_y[32], s_dz[32], s_e2[32];
   __shared__ int64_t s_row[32];
@@ -499,7 +501,7 @@ bool trs_plan(const MlpDesc& m, int B, int sms, int& tr, int& chunk, int64_t& fl
 // further round of tiles costs as much as the first, in proportion to the
 // parameters; the general path pays some seven launches a layer once and its
 // products then fill the GPU.  The line: a 32-row tile per SM (fewer rows where
-// a tile has fewer), 16 rows where the layers average over 12K parameters, and
+// a tile has fewer), 16 rows where the layers average over 15,000 parameters, and
 // none for predictors that are small beside their layer count.  Device time of
 // a step as graph replays on 152 SMs, general path / this one, at or below the
 // line and above it:
@@ -507,8 +509,8 @@ bool trs_plan(const MlpDesc& m, int B, int sms, int& tr, int& chunk, int64_t& fl
 //             80-80-80, d 64    338 / 284 at 16,384
 //   32 rows   128, d 64         70 / 46 at 4864       76 / 80 at 6144
 //             128-128-128, d 64 215 / 145 at 4864     240 / 307 at 6144
-//             160-160, d 64     175 / 138 at 4864     184 / 282 at 6144
-//   16 rows   192-96, d 128     135 / 62 at 2048      187 / 290 at 6144 (164 / 135 at 4096)
+//             192-96, d 128     168 / 137 at 4864     187 / 290 at 6144
+//   16 rows   256, d 128        70 / 45 at 2048       82 / 99 at 3072
 //             512, d 64         64 / 61 at 2048       80 / 121 at 3072
 //             256-256, d 64     166 / 121 at 2048     198 / 250 at 3072
 //             1000, d 16 (tiles of 16)  56 / 43 at 1024  96 / 166 at 3072
@@ -520,7 +522,7 @@ int plan_train_f32(const MlpDesc& m, int64_t n_params, int max_batch, int sms, i
   trs_plan(m, INT_MAX, sms, tr, chunk, floats);  // tr: the rows of a tile of a large batch
   const int64_t layers = m.n_layers;
   const bool small = layers > 1 && n_params <= 1200 * layers * layers;
-  const int line = small ? INT_MAX : std::min(tr, n_params <= 12 * 1024 * layers ? 32 : 16) * sms;
+  const int line = small ? INT_MAX : std::min(tr, n_params <= 15000 * layers ? 32 : 16) * sms;
   const int64_t ctas = std::min<int64_t>(sms, (std::min(max_batch, line) + 3) / 4);
   *part_floats = ctas * (n_params + 2);
   return line;
