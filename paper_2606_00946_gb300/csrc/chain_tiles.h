@@ -1,6 +1,6 @@
 // Where a CTA of the one-launch training step (k_tr_chain) stages the
 // transposed tile of a product for its bulk stores, as a plain function that
-// the kernel calls and a host check goes through (tests/test_chain_tiles.py).
+// the launch lays out and a host check goes through (tests/test_chain_tiles.py).
 #pragma once
 
 #if defined(__CUDACC__)

@@ -807,6 +807,7 @@ struct ChainPhase {
   int drop_h;          // as TrJob's
   uint16_t* mask;      // written by TE_FWD, read by TE_DX
   float* colpart;
+  int stage[2];        // bytes: where each rank stages the transposed tile, in both operand copies
 };
 
 struct ChainArgs {
@@ -967,6 +968,11 @@ __global__ void __launch_bounds__(kChainT, 1) k_tr_chain(const __grid_constant__
         if (P.epi == TE_FWD_OUT) E.s_w[t] = round_bf16(__ldg(a.wL + n0 + t));
       }
       const int cw = NT / 4, cbeg = cq * cw, own0 = chain::first_block(rank, NT);
+      // the transposed tile for its bulk stores takes K-blocks of the operand
+      // just read that the other rank does not write for the next product (it
+      // may be at that epilogue already); this one writes there only in its
+      // own next epilogue, after the stores have read the tile
+      uint8_t* S2 = A + (rank ? P.stage[1] : P.stage[0]);
       uint16_t* mask = P.mask + j + (int64_t)(n0 >> 4) * a.R;
       const uint32_t bits = P.epi == TE_DX ? mask[(int64_t)(cbeg >> 4) * a.R] : 0u;
       if (tid == 0) bulk_commit_wait_read();  // the last product's stores have read S2
@@ -980,12 +986,6 @@ __global__ void __launch_bounds__(kChainT, 1) k_tr_chain(const __grid_constant__
       const bool send = CL > 1 && P.feeds;
       const ClusterRow row{P.feeds ? S1 : nullptr, send ? map_cluster(S1, (uint32_t)rank ^ 1u) : 0,
                            send ? map_cluster(sb, (uint32_t)rank ^ 1u) : 0};
-      // the transposed tile for its bulk stores takes K-blocks of the operand
-      // just read that the other rank does not write for the next product (it
-      // may be at that epilogue already); this one writes there only in its
-      // own next epilogue, after the stores have read the tile
-      const int s2 = chain::stage_block(CL, rank, NT, p + 1 < a.n ? a.ph[p + 1].NT : NT);
-      uint8_t* S2 = A + (size_t)(p & 1) * a.a_bytes + (size_t)s2 * kM * 128;
       if (P.epi == TE_FWD) {
         uint64_t h1 = 0;
         const bool drop = P.drop_h > 0;
@@ -1929,6 +1929,10 @@ cudaError_t run_train_fast(Ctx& c, int B, const int32_t* idx, int opt, float lr,
     if (e != cudaSuccess) return e;
   }
   if (chain) {
+    for (int p = 0; p < ca.n; ++p)
+      for (int r = 0; r < 2; ++r)
+        ca.ph[p].stage[r] = (p & 1) * cp.a_bytes +
+                            chain::stage_block(cp.CL, r, ca.ph[p].NT, ca.ph[p + (p + 1 < ca.n)].NT) * kM * 128;
     ca.CL = cp.CL;
     ca.a_bytes = cp.a_bytes;
     ca.stages = cp.stages;
