@@ -19,7 +19,7 @@ const char* const kTraceNames[TR_COUNT] = {
     "ring_append", "publish", "train_gather", "gemm_fwd", "loss_grad", "gemm_dw", "reduce_dw",
     "colsum_db", "gemm_dx", "optimizer", "memset", "score_tc", "features", "publish_tc",
     "hash_screen", "probe_screen", "probe_walk", "gemm_tc_fwd", "gemm_tc_dw", "gemm_tc_dx", "prefix_index",
-    "index_insert", "guards", "ring_bounds", "replay_admit", "train_step", "route_seq"};
+    "index_insert", "guards", "ring_bounds", "replay_admit", "train_step", "route_seq", "walk_order"};
 }
 
 struct ls_ctx {
@@ -601,10 +601,12 @@ int route_impl(ls_ctx* h, int32_t n_req, const int32_t* tok, const int64_t* tok_
                                                   : simt_selects(c.mlp, n_req, c.n_inst, c.sms));
   float* scores = scores_opt ? scores_opt : (fused_select ? nullptr : c.scores);
   if (c.use_index) {
-    int launches = 1;
-    LS_CK(traced(c, TR_PREFIX_INDEX, launches, s, [&] {
+    const bool sorted = prefix_index_sorts(n_req, c.gW, c.sms);
+    if (sorted)
+      LS_CK(traced(c, TR_WALK_ORDER, 1, s, [&] { return launch_walk_order(n_req, tok_off, c.order, s); }));
+    LS_CK(traced(c, TR_PREFIX_INDEX, 1, s, [&] {
       return launch_prefix_index(n_req, tok, tok_off, c.gkeys, c.gmask, c.gW, (uint64_t)(c.gslots - 1), c.n_inst,
-                                 hits, c.order, c.sms, c.st, &launches, s);
+                                 hits, sorted ? c.order : nullptr, c.sms, c.st, s);
     }));
   } else if (c.cfg.prefix_mode == LS_PREFIX_FUSED) {
     LS_CK(traced(c, TR_PREFIX, 1, s, [&] {

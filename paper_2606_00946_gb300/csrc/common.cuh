@@ -126,7 +126,7 @@ enum TraceId {
   TR_GATHER, TR_GEMM_FWD, TR_LOSS, TR_GEMM_DW, TR_REDUCE, TR_COLSUM, TR_GEMM_DX, TR_OPT,
   TR_MEMSET, TR_SCORE_TC, TR_NORM_ROWS, TR_PUBLISH_TC, TR_HASH_BATCH, TR_SCREEN, TR_WALK,
   TR_GEMM_TC_FWD, TR_GEMM_TC_DW, TR_GEMM_TC_DX, TR_PREFIX_INDEX, TR_INDEX_INSERT,
-  TR_GUARDS, TR_BOUNDS, TR_REPLAY, TR_TRAIN_STEP, TR_ROUTE_SEQ, TR_COUNT
+  TR_GUARDS, TR_BOUNDS, TR_REPLAY, TR_TRAIN_STEP, TR_ROUTE_SEQ, TR_WALK_ORDER, TR_COUNT
 };
 extern const char* const kTraceNames[TR_COUNT];
 
@@ -294,10 +294,9 @@ inline bool capturing(cudaStream_t s) {
   return cudaStreamIsCapturing(s, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
 }
 
-// Launches bracketed by trace events (skipped while the stream is being
-// captured); f may change n_launch, their number, which is read after it.
+// Launch bracketed by trace events (skipped while the stream is being captured).
 template <class F>
-cudaError_t traced(Ctx& c, int id, const int& n_launch, cudaStream_t s, F&& f) {
+cudaError_t traced(Ctx& c, int id, int n_launch, cudaStream_t s, F&& f) {
   const int t = c.tracer.on && !capturing(s) ? c.tracer.begin(s) : -1;
   const cudaError_t e = f();
   c.tracer.end(t, id, n_launch, s);
@@ -583,7 +582,10 @@ cudaError_t run_train_f32(Ctx& c, int batch, const int32_t* idx, int opt, float 
 void set_last_error(const char* msg);  // sets the text ls_last_error() returns
 cudaError_t launch_prefix_index(int n_req, const int32_t* tok, const int64_t* tok_off, const uint64_t* gkeys,
                                 const uint64_t* gmask, int W, uint64_t gmask_slots, int n_inst, int32_t* hits,
-                                uint32_t* order, int sms, DevState* st, int* launches, cudaStream_t s);
+                                const uint32_t* order, int sms, DevState* st, cudaStream_t s);
+// Whether a batch's walk takes its requests in the order of launch_walk_order.
+bool prefix_index_sorts(int n_req, int W, int sms);
+cudaError_t launch_walk_order(int n_req, const int64_t* tok_off, uint32_t* order, cudaStream_t s);
 cudaError_t launch_index_insert(const uint64_t* keys, const int64_t* key_off, int n_inst, int64_t n_keys,
                                 uint64_t* gkeys, uint64_t* gmask, int W, uint64_t gmask_slots, int32_t* counts,
                                 int64_t max_keys, bool cleared, int* err, int sms, cudaStream_t s);

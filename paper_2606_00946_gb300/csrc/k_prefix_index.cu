@@ -566,21 +566,56 @@ __global__ void __launch_bounds__(256) k_index_insert(const uint64_t* __restrict
 
 int index_words(int max_instances) { return max_instances <= 64 ? 1 : max_instances <= 128 ? 2 : max_instances <= 256 ? 4 : max_instances <= 512 ? 8 : 0; }
 
+namespace {
+using WalkKernel = void (*)(int, const int32_t*, const int64_t*, const uint64_t*, const uint64_t*, uint64_t, int,
+                            int32_t*, DevState*, const uint32_t*);
+WalkKernel walk_kernel(int W) {
+  switch (W) {
+    case 1: return k_prefix_index<1>;
+    case 2: return k_prefix_index<2>;
+    case 4: return k_prefix_index<4>;
+    case 8: return k_prefix_index<8>;
+  }
+  return nullptr;
+}
+
+// A CTA of eight or four warps per request while that many CTAs fit.
+bool walk_by_cta(int n_req, int W, int sms) { return n_req <= 8 * sms && (W <= 4 || n_req <= sms); }
+
+// CTAs of the walk by warps that are resident at once.
+int walk_resident(int W, int sms) {
+  static int resident[9] = {};
+  if (!resident[W]) {
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_kernel(W), kNT, 0) != cudaSuccess || per_sm < 1) {
+      cudaGetLastError();
+      per_sm = 1;
+    }
+    resident[W] = per_sm;
+  }
+  return sms * resident[W];
+}
+
+int walk_ctas(int n_req) { return (n_req + kNT / 32 - 1) / (kNT / 32); }  // a warp per request
+}  // namespace
+
+// More requests than warps at once: the long ones first (8192 prompts of 8k to
+// 32k tokens over 64 instances: a route took 334 us in order, 318 so).
+bool prefix_index_sorts(int n_req, int W, int sms) {
+  return walk_kernel(W) && !walk_by_cta(n_req, W, sms) && walk_resident(W, sms) < walk_ctas(n_req);
+}
+
+cudaError_t launch_walk_order(int n_req, const int64_t* tok_off, uint32_t* order, cudaStream_t s) {
+  return launch_chained(k_walk_order, dim3(1), dim3(1024), 0, s, 1, n_req, tok_off, order);
+}
+
 cudaError_t launch_prefix_index(int n_req, const int32_t* tok, const int64_t* tok_off, const uint64_t* gkeys,
                                 const uint64_t* gmask, int W, uint64_t gmask_slots, int n_inst, int32_t* hits,
-                                uint32_t* order, int sms, DevState* st, int* launches, cudaStream_t s) {
+                                const uint32_t* order, int sms, DevState* st, cudaStream_t s) {
   if (n_req <= 0) return cudaSuccess;
-  void (*k)(int, const int32_t*, const int64_t*, const uint64_t*, const uint64_t*, uint64_t, int, int32_t*,
-            DevState*, const uint32_t*) = nullptr;
-  switch (W) {
-    case 1: k = k_prefix_index<1>; break;
-    case 2: k = k_prefix_index<2>; break;
-    case 4: k = k_prefix_index<4>; break;
-    case 8: k = k_prefix_index<8>; break;
-    default: return cudaErrorInvalidValue;
-  }
-  // a CTA of eight or four warps per request while that many CTAs fit
-  if (n_req <= 8 * sms && (W <= 4 || n_req <= sms)) {
+  const WalkKernel k = walk_kernel(W);
+  if (!k) return cudaErrorInvalidValue;
+  if (walk_by_cta(n_req, W, sms)) {
     void (*c)(const int32_t*, const int64_t*, const uint64_t*, const uint64_t*, uint64_t, int, int32_t*, DevState*) =
         nullptr;
     const bool wide = n_req <= 4 * sms;
@@ -595,27 +630,9 @@ cudaError_t launch_prefix_index(int n_req, const int32_t* tok, const int64_t* to
   }
   // as many warps as are resident at once (they then take requests from the
   // counter); with no state to keep the counter in, one warp per request
-  static int resident[9] = {};
-  if (!resident[W]) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kNT, 0) != cudaSuccess || per_sm < 1) {
-      cudaGetLastError();
-      per_sm = 1;
-    }
-    resident[W] = per_sm;
-  }
-  const int want = (n_req + kNT / 32 - 1) / (kNT / 32);
-  const int grid = std::max(1, std::min(want, st ? sms * resident[W] : sms * 16));
-  // more requests than warps at once: the long ones first (8192 prompts of 8k
-  // to 32k tokens over 64 instances: a route took 334 us in order, 318 so)
-  const bool sorted = order && grid < want;
-  *launches = sorted ? 2 : 1;
-  if (sorted) {
-    const cudaError_t e = launch_chained(k_walk_order, dim3(1), dim3(1024), 0, s, 1, n_req, tok_off, order);
-    if (e != cudaSuccess) return e;
-  }
+  const int grid = std::max(1, std::min(walk_ctas(n_req), st ? walk_resident(W, sms) : sms * 16));
   return launch_chained(k, dim3(grid), dim3(kNT), 0, s, 1, n_req, tok, tok_off, gkeys, gmask, gmask_slots, n_inst,
-                        hits, st, (const uint32_t*)(sorted ? order : nullptr));
+                        hits, st, order);
 }
 
 cudaError_t launch_index_insert(const uint64_t* keys, const int64_t* key_off, int n_inst, int64_t n_keys,

@@ -66,9 +66,9 @@ def test_hits_equal_the_two_phase_kernels(n_req, n_inst, max_len, shift):
         r.close()
 
 
-def test_the_trace_counts_the_sort():
-    """A traced route's launches: the walk alone, or the sort by length before it."""
-    for n_req, want in ((64, 1), (1300, 1), (6000, 2)):
+def test_the_trace_lists_the_sort():
+    """A traced route's launches: the walk alone, or the sort by length and the walk."""
+    for n_req, want in ((64, 0), (1300, 0), (6000, 1)):
         r = H.Router([16, 64, 1], 10, 0, "bf16", max_instances=4, max_requests=n_req, max_keys_per_instance=64,
                      max_batch_tokens=16 * n_req, ring_capacity=16, max_train_batch=64)
         r.set_normalizer(torch.zeros(16, device="cuda"), torch.ones(16, device="cuda"))
@@ -80,5 +80,6 @@ def test_the_trace_counts_the_sort():
         assert L.ls_trace_enable(r.h, True) == L.LS_OK
         r.route(tok, off, torch.zeros(n_req, 0, device="cuda"), 4)
         rc, entries = L.ls_trace_read(r.h)
-        assert rc == L.LS_OK and entries["prefix_index"][0] == want, (n_req, entries)
+        assert rc == L.LS_OK and entries["prefix_index"][0] == 1, (n_req, entries)
+        assert entries.get("walk_order", (0,))[0] == want, (n_req, entries)
         r.close()
